@@ -341,13 +341,28 @@ int dpm_server_submit(dpm_server *server, int geometry_id, const dpm_source *src
    resubmit the requests to a new one (the old slots stay phantoms of the
    context until dpm_free_phantom or dpm_destroy). */
 int dpm_server_round(dpm_server *server, int *n_completed);
+/* The same round in two halves, so that the host can take requests in while the
+   GPU works: dpm_server_round_begin() admits, chooses and queues the round's
+   work without waiting (*n_jobs receives its requests, 0 when there is nothing
+   to run; DPM_ESTATE if a round is in flight on the context), dpm_server_round_ready()
+   says whether that work has finished, and dpm_server_round_end() waits for it
+   and takes the results in as dpm_server_round() does (nothing to do without a
+   round in flight).  In between, requests may be submitted and asked about, and
+   dpm_server_admit() gives pending ones their slots (a slot's copies queue up
+   behind the round), so that the next round starts without that work; other
+   calls on the context belong before or after.  n_jobs and n_completed may be
+   NULL. */
+int dpm_server_round_begin(dpm_server *server, int *n_jobs);
+int dpm_server_round_ready(dpm_server *server, int *ready);
+int dpm_server_round_end(dpm_server *server, int *n_completed);
+int dpm_server_admit(dpm_server *server);
 /* A request's state and statistics; DPM_EINVAL for a bad id. */
 int dpm_server_status(dpm_server *server, int request_id, dpm_request_status *status);
 typedef struct {
     int n_pending;             /* submitted, not yet admitted */
     int n_active;              /* admitted, not done */
     int n_done;                /* done, not yet released */
-    int max_active;            /* most requests active in one round */
+    int max_active;            /* most requests active at once */
     uint64_t n_rounds;         /* rounds that ran a batch */
     uint64_t n_completed;      /* requests that reached the target */
     uint64_t histories;        /* histories transported by all rounds */

@@ -261,6 +261,42 @@ int ctx_run_params_f64(dpm_ctx *c, PhantomState *p, const dpm_source *src, uint6
   return fill_run_params(c, p, src, first, n, seed, physics_flags, c->dt64, (const double *)p->d_mumax64, R);
 }
 
+int ctx_dmax_launch(dpm_ctx *c, DmaxOut &o, const int *ids, int n) {
+  cudaSetDevice(c->device);
+  std::vector<PhantomState *> ps(n);
+  for (int i = 0; i < n; ++i) {
+    ps[i] = get_phantom(c, ids[i]);
+    if (!ps[i]) return fail(c, DPM_EINVAL, "bad phantom id");
+    if (!ps[i]->d_dmax) {
+      int rc = dalloc(c, &ps[i]->d_dmax, size_t(4));
+      if (rc) return rc;
+    }
+  }
+  if (n > o.cap) {
+    dfree(c, o.d);
+    o.d = nullptr;
+    o.cap = 0;
+    int rc = dalloc(c, &o.d, size_t(3) * size_t(n));
+    if (rc) return rc;
+    o.cap = n;
+  }
+  // every request's result lands in one device array: one copy back
+  for (int i = 0; i < n; ++i) {
+    PhantomState *p = ps[i];
+    launch_dmax(p->d_S1, p->d_Q, p->d_rho, p->V, double(p->n_total), double(p->b_total), p->dx * p->dy * p->dz,
+                p->d_dmax, o.d + 3 * i, c->sm_count, c->stream);
+  }
+  CUDA_TRY(c, cudaGetLastError());
+  return DPM_OK;
+}
+
+int ctx_dmax_read(dpm_ctx *c, const DmaxOut &o, int n, double *out) {
+  const int src = dpm_sync(c);
+  if (src == DPM_ECUDA) return src;
+  if (n > 0) CUDA_TRY(c, cudaMemcpy(out, o.d, 3 * sizeof(double) * size_t(n), cudaMemcpyDeviceToHost));
+  return src;
+}
+
 }  // namespace dpm
 
 extern "C" {
@@ -307,7 +343,8 @@ void dpm_destroy(dpm_ctx *c) {
   free_tables(c);
   queue_free(c->queue);
   dfree(c, c->d_jobs);
-  dfree(c, c->d_dmax_out);
+  dfree(c, c->dmax.d);
+  dfree(c, c->round_dmax.d);
   dfree(c, c->d_batch_counters);
   for (cudaEvent_t e : c->batch_ev) cudaEventDestroy(e);
   if (c->batch_exec) cudaGraphExecDestroy(c->batch_exec);
@@ -676,35 +713,8 @@ int dpm_run(dpm_ctx *c, int id, const dpm_source *src, uint64_t first, uint64_t 
 int dpm_dmax_sigma(dpm_ctx *c, const int *ids, int n, double *out) {
   if (!c) return DPM_EINVAL;
   if (n < 0 || (n > 0 && (!ids || !out))) return fail(c, DPM_EINVAL, "bad arguments");
-  cudaSetDevice(c->device);
-  std::vector<PhantomState *> ps(n);
-  for (int i = 0; i < n; ++i) {
-    ps[i] = get_phantom(c, ids[i]);
-    if (!ps[i]) return fail(c, DPM_EINVAL, "bad phantom id");
-    if (!ps[i]->d_dmax) {
-      int rc = dalloc(c, &ps[i]->d_dmax, size_t(4));
-      if (rc) return rc;
-    }
-  }
-  if (n > c->dmax_cap) {
-    dfree(c, c->d_dmax_out);
-    c->d_dmax_out = nullptr;
-    c->dmax_cap = 0;
-    int rc = dalloc(c, &c->d_dmax_out, size_t(3) * size_t(n));
-    if (rc) return rc;
-    c->dmax_cap = n;
-  }
-  // every request's result lands in one device array: one copy back
-  for (int i = 0; i < n; ++i) {
-    PhantomState *p = ps[i];
-    launch_dmax(p->d_S1, p->d_Q, p->d_rho, p->V, double(p->n_total), double(p->b_total), p->dx * p->dy * p->dz,
-                p->d_dmax, c->d_dmax_out + 3 * i, c->sm_count, c->stream);
-  }
-  CUDA_TRY(c, cudaGetLastError());
-  const int src = dpm_sync(c);
-  if (src == DPM_ECUDA) return src;
-  if (n > 0) CUDA_TRY(c, cudaMemcpy(out, c->d_dmax_out, 3 * sizeof(double) * size_t(n), cudaMemcpyDeviceToHost));
-  return src;
+  const int rc = ctx_dmax_launch(c, c->dmax, ids, n);
+  return rc ? rc : ctx_dmax_read(c, c->dmax, n, out);
 }
 
 int dpm_sync(dpm_ctx *c) {

@@ -54,6 +54,12 @@ struct PhantomState {
   uint64_t folded_launches = 0;
 };
 
+// Device results of D_max queries, three doubles for each of up to `cap` phantoms.
+struct DmaxOut {
+  double *d = nullptr;
+  int cap = 0;
+};
+
 }  // namespace dpm
 
 struct dpm_ctx {
@@ -78,8 +84,9 @@ struct dpm_ctx {
   dpm::QueueState queue;
   // batches
   dpm::DevJob *d_jobs = nullptr;               // job table, kMaxJobs entries
-  double *d_dmax_out = nullptr;                // dpm_dmax_sigma results, 3 per phantom [dmax_cap]
-  int dmax_cap = 0;
+  dpm::DmaxOut dmax;        // dpm_dmax_sigma results
+  dpm::DmaxOut round_dmax;  // those of the server round in flight
+  const void *round_of = nullptr;  // the server whose round is in flight
   unsigned long long *d_batch_counters = nullptr;  // [kCounterSlots]
   std::vector<cudaEvent_t> batch_ev;           // start/end pairs since the last dpm_batch_stats
   double batch_folded_ms = 0;                  // times of pairs retired early (see kMaxPendingEvents)
@@ -106,6 +113,10 @@ int ctx_alloc(dpm_ctx *c, void **p, size_t bytes);
 // Batch structure of a run of n histories in (at most) n_batches batches:
 // makes sure the phantom has B slabs and uploads 1/n_b; returns bs and B.
 int ctx_prepare_batches(dpm_ctx *c, PhantomState *p, uint64_t n, int n_batches, uint64_t &bs, int &B);
+// dpm_dmax_sigma() in two halves: the kernels queued on the stream, and the wait
+// with the read-back of their n results.
+int ctx_dmax_launch(dpm_ctx *c, DmaxOut &o, const int *ids, int n);
+int ctx_dmax_read(dpm_ctx *c, const DmaxOut &o, int n, double *out);
 // With the context's device current: load the module holding the scratch of
 // dpm_run_noalloc() and the queue kernels (dpm_noalloc.cu).
 int noalloc_setup(std::string &err);

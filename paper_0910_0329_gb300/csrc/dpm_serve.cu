@@ -59,6 +59,7 @@ struct dpm_server {
   std::vector<Request> req;          // by request id
   std::deque<int> pending;           // ids in submission order
   std::vector<int> active;           // ids in admission order
+  std::vector<int> chosen;           // ids of the round in flight
   std::vector<Geometry> geom;        // by geometry phantom id
   std::vector<int> slot_geometry;    // by phantom id: the geometry a slot copies (-1: not a slot)
   uint64_t used = 0;                 // device bytes held by slots
@@ -198,6 +199,7 @@ int dpm_server_create(dpm_ctx *ctx, const dpm_serve_opts *opts, dpm_server **out
 void dpm_server_destroy(dpm_server *s) {
   if (!s) return;
   // the slots stay loaded phantoms of the context (freed with it)
+  if (!s->chosen.empty()) s->ctx->round_of = nullptr;  // a round in flight ends unread
   delete s;
 }
 
@@ -217,11 +219,9 @@ int dpm_server_submit(dpm_server *s, int geometry_id, const dpm_source *src, uin
   return DPM_OK;
 }
 
-int dpm_server_round(dpm_server *s, int *n_completed) {
-  if (!s) return DPM_EINVAL;
-  if (n_completed) *n_completed = 0;
+// Admit pending requests in submission order while slots and room allow.
+static int admit(dpm_server *s) {
   int rc = DPM_OK;
-  // admit in submission order while slots and room allow
   for (auto it = s->pending.begin(); it != s->pending.end() && int(s->active.size()) < s->o.max_active;) {
     Request &r = s->req[size_t(*it)];
     const int slot = take_slot(s, r.geometry, rc);
@@ -236,8 +236,22 @@ int dpm_server_round(dpm_server *s, int *n_completed) {
     s->active.push_back(*it);
     it = s->pending.erase(it);
   }
-  if (s->active.empty()) return DPM_OK;
   s->info.max_active = std::max(s->info.max_active, int(s->active.size()));
+  return DPM_OK;
+}
+
+int dpm_server_admit(dpm_server *s) {
+  if (!s) return DPM_EINVAL;
+  return admit(s);
+}
+
+int dpm_server_round_begin(dpm_server *s, int *n_jobs) {
+  if (!s) return DPM_EINVAL;
+  if (n_jobs) *n_jobs = 0;
+  if (s->ctx->round_of) return srv_fail(s, DPM_ESTATE, "a round is in flight on the context");
+  int rc = admit(s);
+  if (rc) return rc;
+  if (s->active.empty()) return DPM_OK;
   // the oldest requests whose next chunks fit the budget (the oldest always)
   std::vector<uint64_t> want(s->active.size());
   for (size_t i = 0; i < s->active.size(); ++i) want[i] = s->req[size_t(s->active[i])].next_n;
@@ -259,8 +273,33 @@ int dpm_server_round(dpm_server *s, int *n_completed) {
   dpm_run_opts ro{};
   ro.n_batches = s->o.n_batches;
   if ((rc = dpm_run_batch(s->ctx, jobs.data(), int(jobs.size()), &ro))) return rc;
+  if ((rc = ctx_dmax_launch(s->ctx, s->ctx->round_dmax, slots.data(), int(slots.size())))) return rc;
+  s->chosen.swap(chosen);
+  s->ctx->round_of = s;
+  if (n_jobs) *n_jobs = k;
+  return DPM_OK;
+}
+
+int dpm_server_round_ready(dpm_server *s, int *ready) {
+  if (!s) return DPM_EINVAL;
+  if (!ready) return srv_fail(s, DPM_EINVAL, "null output");
+  cudaSetDevice(s->ctx->device);
+  const cudaError_t e = s->chosen.empty() ? cudaSuccess : cudaStreamQuery(s->ctx->stream);
+  *ready = e != cudaErrorNotReady;  // an error is reported by dpm_server_round_end()
+  if (e != cudaSuccess) cudaGetLastError();
+  return DPM_OK;
+}
+
+int dpm_server_round_end(dpm_server *s, int *n_completed) {
+  if (!s) return DPM_EINVAL;
+  if (n_completed) *n_completed = 0;
+  if (s->chosen.empty()) return DPM_OK;
+  std::vector<int> chosen;
+  chosen.swap(s->chosen);
+  s->ctx->round_of = nullptr;
+  int rc = DPM_OK;
   std::vector<double> res(3 * chosen.size());
-  if ((rc = dpm_dmax_sigma(s->ctx, slots.data(), int(slots.size()), res.data()))) return rc;
+  if ((rc = ctx_dmax_read(s->ctx, s->ctx->round_dmax, int(chosen.size()), res.data()))) return rc;
   // the round's device status (a queue overflow or a timed-out wait is an
   // error of the round) and release of its timing events
   dpm_run_stats st{};
@@ -292,6 +331,14 @@ int dpm_server_round(dpm_server *s, int *n_completed) {
   }
   if (n_completed) *n_completed = done;
   return DPM_OK;
+}
+
+int dpm_server_round(dpm_server *s, int *n_completed) {
+  if (!s) return DPM_EINVAL;
+  if (n_completed) *n_completed = 0;
+  int rc = DPM_OK;
+  if (s->chosen.empty() && (rc = dpm_server_round_begin(s, nullptr))) return rc;
+  return dpm_server_round_end(s, n_completed);
 }
 
 int dpm_server_status(dpm_server *s, int request_id, dpm_request_status *out) {

@@ -125,6 +125,10 @@ _SIGS = {
     "dpm_server_destroy": (None, [_P]),
     "dpm_server_submit": (C.c_int, [_P, C.c_int, C.POINTER(dpm_source), C.c_uint64, C.POINTER(C.c_int)]),
     "dpm_server_round": (C.c_int, [_P, C.POINTER(C.c_int)]),
+    "dpm_server_round_begin": (C.c_int, [_P, C.POINTER(C.c_int)]),
+    "dpm_server_round_ready": (C.c_int, [_P, C.POINTER(C.c_int)]),
+    "dpm_server_round_end": (C.c_int, [_P, C.POINTER(C.c_int)]),
+    "dpm_server_admit": (C.c_int, [_P]),
     "dpm_server_status": (C.c_int, [_P, C.c_int, C.POINTER(dpm_request_status)]),
     "dpm_server_info_get": (C.c_int, [_P, C.POINTER(dpm_server_info)]),
     "dpm_server_slot_bytes": (C.c_int, [_P, C.c_int, C.POINTER(C.c_uint64)]),
@@ -364,6 +368,25 @@ class Server:
         done = C.c_int(0)
         self._chk(lib().dpm_server_round(self.h, C.byref(done)))
         return done.value
+
+    def round_begin(self) -> int:
+        """Queue a round's work without waiting; the requests in it."""
+        n = C.c_int(0)
+        self._chk(lib().dpm_server_round_begin(self.h, C.byref(n)))
+        return n.value
+
+    def round_ready(self) -> bool:
+        ready = C.c_int(0)
+        self._chk(lib().dpm_server_round_ready(self.h, C.byref(ready)))
+        return bool(ready.value)
+
+    def round_end(self) -> int:
+        done = C.c_int(0)
+        self._chk(lib().dpm_server_round_end(self.h, C.byref(done)))
+        return done.value
+
+    def admit(self):
+        self._chk(lib().dpm_server_admit(self.h))
 
     def status(self, rid) -> dict:
         st = dpm_request_status()

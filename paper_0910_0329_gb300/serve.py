@@ -144,17 +144,27 @@ class Server:
         todo = sorted(requests, key=lambda r: r.arrival)
         waiting = {}  # library request id -> Request
         i = 0
-        while i < len(todo) or waiting:
-            now = clock()
+
+        def arrivals():
+            nonlocal i
+            now, k = clock(), i
             while i < len(todo) and todo[i].arrival <= now:
                 r = todo[i]
                 waiting[self.srv.submit(self.template[r.geometry], r.source, self.seed_base + r.rid)] = r
                 i += 1
+            return now, i > k
+
+        while i < len(todo) or waiting:
+            now, _ = arrivals()
             if waiting:
-                before = self.srv.info()["n_rounds"]
-                self.srv.round()
-                info = self.srv.info()
-                if info["n_rounds"] == before and info["n_pending"]:
+                # requests that arrive while the round is on the GPU get their
+                # slots meanwhile
+                ran = self.srv.round_begin()
+                while i < len(todo) and not self.srv.round_ready():
+                    if arrivals()[1]:
+                        self.srv.admit()
+                self.srv.round_end()
+                if not ran and self.srv.info()["n_pending"]:
                     # nothing active and still nothing admissible, with every
                     # released slot free to go
                     raise RuntimeError("a request does not fit the HBM budget")
