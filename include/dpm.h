@@ -120,11 +120,11 @@ typedef struct {
     int block_size;    /* per-history kernel: threads per block (multiple of 32; 0 = 128).
                           The queue kernel always runs blocks of 128 threads (it schedules
                           per warp); its size is set by blocks_per_sm */
-    int blocks_per_sm; /* queue kernel: resident blocks per SM (0 = as many as fit, 8) */
+    int blocks_per_sm; /* queue kernel: resident blocks per SM (0 = as many as fit, 6) */
     int queue_log2;    /* queue kernel: log2 of each queue shard's capacity (7..20; 0 = 15 for
                           an electron-beam dpm_run, 14 otherwise) */
-    int refill_min;    /* queue kernel: idle lanes before a warp refills (1..32; 0 = 24 for
-                          photon warps, 12 for electron warps) */
+    int refill_min;    /* queue kernel: idle lanes before a warp takes particles from its
+                          stash (1..32; 0 = 2) */
     double timeout_s;  /* bound on any device wait (default 20 s) */
     int physics_flags; /* DPM_NO_HARD: no Moller/bremsstrahlung events; DPM_NO_MSC: no
                           elastic deflections (test and ablation switches; 0 = full physics);
@@ -140,13 +140,9 @@ typedef struct {
                           (about 10 % slower); 0 = those counts read 0.  The energy
                           counters and the tally are the same either way.  The per-history
                           kernels always count. */
-    int refill_pause;  /* queue kernel: a warp with particles whose refill found nothing
-                          waits 128 steps before it tries again (1), or tries on every
-                          step (-1); 0 = automatic: the pause for launches of at most
-                          1.6e7 photon-beam histories or 2e6 electron-beam histories
-                          (a batch launch: its jobs' histories, an electron history
-                          counting 8), where it shortens the end of the launch, and none
-                          above, where it costs about 1.5 %; none either with queue
+    int refill_pause;  /* queue kernel: a warp with particles that found none to fetch
+                          waits 128 steps before it looks again (1), or looks on every
+                          step (-1); 0 = automatic: the pause, but none with queue
                           shards below 2^13 slots (queue_log2 < 13, or
                           dpm_run_noalloc's), which need every refill to keep from
                           overflowing.  Scheduling only: the tally is the same either

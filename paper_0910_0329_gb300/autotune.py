@@ -16,9 +16,9 @@ import os
 
 DEFAULT_SPACE = {
     "queue_log2": [12, 13, 14, 15],
-    "blocks_per_sm": [4, 6, 8],
-    "refill_min": [0, 8, 16, 24],  # 0: the library's per-type defaults (24 photon, 12 electron lanes)
-    "refill_pause": [0, -1, 1],  # 0: the library's choice by launch length
+    "blocks_per_sm": [4, 6, 8],  # 6 fit, more are the same
+    "refill_min": [0, 8, 16, 24],  # 0: the library's default (2 lanes)
+    "refill_pause": [0, -1, 1],  # 0: the library's choice by queue size
 }
 DEFAULT_START = {"queue_log2": 14, "blocks_per_sm": 8, "refill_min": 0, "refill_pause": 0}
 

@@ -221,6 +221,9 @@ static int fill_run_params(dpm_ctx *c, PhantomState *p, const dpm_source *src, u
   R.P.dx = Real(p->dx);
   R.P.dy = Real(p->dy);
   R.P.dz = Real(p->dz);
+  R.P.rdx = Real(1) / R.P.dx;
+  R.P.rdy = Real(1) / R.P.dy;
+  R.P.rdz = Real(1) / R.P.dz;
   R.P.mat = p->d_mat;
   R.P.rho = p->d_rho;
   R.P.mu_max = mu_max;

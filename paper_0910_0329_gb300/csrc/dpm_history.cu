@@ -8,6 +8,22 @@
 
 namespace dpm {
 
+// The particle that emission o of p creates: at p's place, with its own random
+// stream.
+template <class Real>
+__device__ __forceinline__ PartT<Real> secondary(const PartT<Real> &p, const EmissionT<Real> &o) {
+  PartT<Real> c = p;
+  c.type = o.type;
+  c.E = o.E;
+  c.u = o.u;
+  c.v = o.v;
+  c.w = o.w;
+  c.id_lo = o.id_lo;
+  c.id_hi = o.id_hi;
+  c.ctr = 0;
+  return c;
+}
+
 // Tally sink with run-length coalescing: consecutive deposits of one thread
 // into the same voxel are summed in a register and issued as one 64-bit
 // atomic add (exact, order-independent fixed point, 2^-32 MeV).  Real: the
@@ -50,13 +66,17 @@ struct HistSinkT {
     }
   }
   __device__ __forceinline__ void escape(Real E) { cnt[C_ESC] += fxc(E); }
-  __device__ __forceinline__ void push(const PartT<Real> &q) {
+  Real held_ = Real(0);
+  __device__ __forceinline__ void hold(Real x) { held_ = x; }
+  __device__ __forceinline__ Real held() const { return held_; }
+  // secondary o of particle p
+  __device__ __forceinline__ void push(const PartT<Real> &p, const EmissionT<Real> &o) {
     ++cnt[C_PUSH];
     if (sp < cap) {
-      stack[sp++] = q;
+      stack[sp++] = secondary(p, o);
     } else {
       err |= ERR_OVERFLOW;
-      cnt[C_ESC] += fxc(q.E + (q.type == POSITRON ? Real(2) * Num<Real>::mc2 : Real(0)));
+      cnt[C_ESC] += fxc(o.E + (o.type == POSITRON ? Real(2) * Num<Real>::mc2 : Real(0)));
     }
   }
   __device__ __forceinline__ void error(int e) { err |= e; }
@@ -83,6 +103,30 @@ __device__ void reduce_counters(const long long *cnt, int err, const RP &R) {
 
 constexpr int kHistStack = 64;
 
+// Transport every particle on the thread's stack, secondaries included.
+template <class Real, class Sink>
+__device__ __forceinline__ void run_stack(const RunParamsT<Real> &R, Sink &s) {
+  while (s.sp > 0) {
+    PartT<Real> q = s.stack[--s.sp];
+    const bool photon = q.type == PHOTON;
+    const uint32_t cap = photon ? kMaxPhotonBlocks : kMaxElectronBlocks;
+    EmissionT<Real> o;
+    for (;;) {
+      o.kind = EM_NONE;
+      const bool alive = (q.type & CHAIN)      ? chain_step(q, R, s, o)
+                         : photon              ? photon_flight(q, R, s, o)
+                                               : electron_step(q, R, s, o);
+      if (o.kind != EM_NONE && settle(q, o, R, s)) s.push(q, o);
+      if (!alive) break;
+      if (q.ctr >= cap) {
+        s.error(ERR_STEPCAP);
+        s.deposit(vox(q, R.P), q.E);
+        break;
+      }
+    }
+  }
+}
+
 // 8 resident blocks of 128 threads cap the registers at 64, as in the queue
 // kernel: the extra spills cost less than the doubled occupancy gains
 // (+26 % on 6 MV, +30 % on 20 MeV electrons against 128 registers).
@@ -103,28 +147,7 @@ __global__ void __launch_bounds__(128, 8) k_history(const __grid_constant__ RunP
     }
     s.sp = 0;
     s.stack[s.sp++] = p;
-    while (s.sp > 0) {
-      PartT<Real> q = s.stack[--s.sp];
-      if (q.type == PHOTON) {
-        int g = 0;
-        while (photon_segment(q, R, s)) {
-          if (++g >= kMaxPhotonSegments) {
-            s.error(ERR_STEPCAP);
-            s.deposit(vox(q, R.P), q.E);
-            break;
-          }
-        }
-      } else {
-        int n = 0;
-        while (electron_step(q, R, s)) {
-          if (++n >= kMaxElectronSteps) {
-            s.error(ERR_STEPCAP);
-            s.deposit(vox(q, R.P), q.E);
-            break;
-          }
-        }
-      }
-    }
+    run_stack(R, s);
     s.flush();
   }
   reduce_counters(s.cnt, s.err, R);
@@ -220,13 +243,16 @@ struct PaperSink {
   // run counters exactly as HistSink keeps them, so that the energy balance
   // of both tallies is the same
   __device__ __forceinline__ void escape(float E) { cnt[C_ESC] += HistSink::fxc(E); }
-  __device__ __forceinline__ void push(const Part &q) {
+  float held_ = 0.f;
+  __device__ __forceinline__ void hold(float x) { held_ = x; }
+  __device__ __forceinline__ float held() const { return held_; }
+  __device__ __forceinline__ void push(const Part &p, const Emission &o) {
     ++cnt[C_PUSH];
     if (sp < cap) {
-      stack[sp++] = q;
+      stack[sp++] = secondary(p, o);
     } else {
       err |= ERR_OVERFLOW;
-      cnt[C_ESC] += HistSink::fxc(q.E + (q.type == POSITRON ? 2.f * kMc2f : 0.f));
+      cnt[C_ESC] += HistSink::fxc(o.E + (o.type == POSITRON ? 2.f * kMc2f : 0.f));
     }
   }
   __device__ __forceinline__ void error(int e) { err |= e; }
@@ -253,28 +279,7 @@ __global__ void __launch_bounds__(128) k_history_paper(const __grid_constant__ R
     }
     s.sp = 0;
     s.stack[s.sp++] = p;
-    while (s.sp > 0) {
-      Part q = s.stack[--s.sp];
-      if (q.type == PHOTON) {
-        int g = 0;
-        while (photon_segment(q, R, s)) {
-          if (++g >= kMaxPhotonSegments) {
-            s.error(ERR_STEPCAP);
-            s.deposit(vox(q, R.P), q.E);
-            break;
-          }
-        }
-      } else {
-        int n = 0;
-        while (electron_step(q, R, s)) {
-          if (++n >= kMaxElectronSteps) {
-            s.error(ERR_STEPCAP);
-            s.deposit(vox(q, R.P), q.E);
-            break;
-          }
-        }
-      }
-    }
+    run_stack(R, s);
     s.flush();
   }
   reduce_counters(s.cnt, s.err, R);

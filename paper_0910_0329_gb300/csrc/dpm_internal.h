@@ -77,6 +77,7 @@ template <class Real>
 struct DevPhantomT {
   int nx, ny, nz;
   Real dx, dy, dz;
+  Real rdx, rdy, rdz;  // 1/dx, 1/dy, 1/dz to the nearest
   const uint8_t *mat;
   const float *rho;
   const Real *mu_max;  // [n_e] photon majorant, 1/cm, on the tables' energy grid

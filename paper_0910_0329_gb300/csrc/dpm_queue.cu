@@ -4,22 +4,44 @@
 // statistically independent paths and execute mostly one at a time (its
 // Sec. 4 diagnosis of the C1060 speed-up).  Here every warp holds particles of
 // ONE type (photons or electrons/positrons) in its lanes, steps them together,
-// and refills lanes that have finished from per-type particle queues;
-// secondaries are pushed to those queues with one atomic per warp.  The
-// physics of a particle is the same code as in the per-history kernel and its
-// random numbers are keyed by its identity, so both kernels produce the same
-// integer tally.
+// and refills lanes that have finished from a stash of its own in shared
+// memory.  The stash is filled 32 particles at a time: with new histories, which
+// all lanes make together, or from per-type particle queues.  Secondaries of
+// the warp's type go to its stash, the others by way of a buffer to the queues.
+// The physics of a particle is the same code as in the per-history kernel and
+// its random numbers are keyed by its identity, so both kernels produce the
+// same integer tally.
 //
-// Queues: for each type, one ring per CTA ("shard") in global memory, SoA, with
-// a sequence number per slot (a producer publishes position p by writing p+1,
+// Queues: for each type, one ring per CTA ("shard") in global memory, with a
+// sequence number per slot (a producer publishes position p by writing p+1,
 // the consumer frees the slot for position p+capacity), so that producers and
 // consumers on different SMs never read a half-written record.  A warp pushes
 // to its CTA's shard and pops from it first, stealing from other shards when it
 // is empty.  The grid alternates between a source phase and a secondary
 // phase (see the scheduler below) so that all SMs run one particle type's
-// code at a time.  The run ends when every started warp is idle, every queue
-// is empty and the source is exhausted.  Every wait is bounded by a time limit read from
-// %globaltimer; on expiry the kernel records an error and returns.
+// code at a time.  The run ends when every started warp is idle (its stash and
+// buffer empty), every queue is empty and the source is exhausted.  Every wait
+// is bounded by a time limit read from %globaltimer; on expiry the kernel
+// records an error and returns.
+//
+// What bounds the kernel: instruction issue, instruction fetch and the latency
+// of table lookups, not memory bandwidth.  Three things follow.
+// - Code size.  The kernel took 276 KB when every secondary was queued where it
+//   is made, every refill was spelled out and the photon interaction stood
+//   after each of two flights; "no instruction" was the leading stall (4.7 of
+//   17 cycles per issue on 6 MV, 5.0 on 20 MeV electrons).  With one copy of
+//   each it takes 83 KB (2.1 and 2.0 cycles).
+// - Full warps.  Lanes that wait for a refill waste issue slots, and a refill
+//   from the device-wide queues costs several L2 round trips.  Taking from the
+//   stash costs some 60 instructions, so it happens at 2 idle lanes: 28.5
+//   (photons) and 28.7 (electrons) of 32 lanes carry particles on 3x10^7 6 MV
+//   histories, against 19.1 and 25.5 with refills from the queues at 24 and 12
+//   idle lanes.
+// - Few instructions per step: see Num<float> and electron_step in
+//   dpm_device.cuh.
+// Transport times, before and with all three: 10^7 6 MV histories 14.6 and
+// 10.1 ms, 5x10^6 20 MeV electrons on the 128^3 blobs 52.4 and 33.2 ms, 2x10^4
+// on the slabs 1.58 and 0.79 ms, 2000 photons of 15 MeV 0.63 and 0.47 ms.
 #include <cuda_runtime.h>
 
 #include "dpm_device.cuh"
@@ -61,46 +83,62 @@ constexpr int kQBlock = 128;
 #define DPM_PHASE_GUARD_SHIFT_E 2
 #endif
 constexpr int kStealProbes = DPM_STEAL_PROBES;
-// Default refill thresholds (idle lanes) of photon and electron warps.  A
-// photon lane's particle is short-lived and starting histories is costly, so
-// photon warps gather more idle lanes per refill (6 MV, 10^7 histories:
-// 16, 20, 22, 24 and 28 lanes measured 6.65, 6.86, 6.94, 7.01 and 6.99 x 10^8
-// histories/s; electron beams within 0.3 % of each other).
+// Idle lanes at which a warp takes particles from its stash, by particle type:
+// 1 to 4 measured within 1 % of each other, 8 and 12 1 to 2 % slower.
 #ifndef DPM_REFILL_MIN_G
-#define DPM_REFILL_MIN_G 24
+#define DPM_REFILL_MIN_G 2
 #endif
 #ifndef DPM_REFILL_MIN_E
-#define DPM_REFILL_MIN_E 12
+#define DPM_REFILL_MIN_E 2
 #endif
-// Refill pause (kernels with kPause): a warp with particles waits this many
-// steps, after a refill that added none, before it tries again.  A failed
-// refill costs several dependent L2 round trips (the home shard, then the
-// steal probes).  Where the queues have run dry, at the end of a launch, the
-// sparse warps that carry the last particles paid that on every step, and
-// the end of a launch took longer than its share of histories: a 6 MV launch
-// of 10^6 histories takes 2.41 ms without the pause and 2.11 ms with it, one
-// of 10^7 1.5 % less time.  In the middle of a long launch the pause costs
-// about 1.5 % (6 MV 5x10^7: +1.5 %; 20 MeV electrons at 10^7: +0.7 to
-// +0.9 %), so a launch takes it when it is short (queue_launch).  Pauses of
-// 8 to 128 steps measured; the longer ones were faster.
+// Idle lanes at which a warp with an empty stash looks for more (4 and 16:
+// -4 and -1 %).
+#ifndef DPM_FETCH_MIN
+#define DPM_FETCH_MIN 8
+#endif
+// Records of a warp's stash and of its out buffer, which always has room for a
+// step's 32.  Larger ones (48, 64) measured the same.
+constexpr int kStash = 32;
+constexpr int kOut = 48;
+// Fetch pause: a warp with particles waits this many steps, after it found no
+// work for its stash, before it looks again.  A look costs several dependent L2
+// round trips, and in the phase of the other type, or at the end of a launch,
+// it finds nothing for hundreds of steps (10^7 20 MeV electrons on the blobs
+// -5 %, 3x10^7 6 MV histories -2 % against no pause).
 #ifndef DPM_REFILL_COOLDOWN
 #define DPM_REFILL_COOLDOWN 128
 #endif
-// Random draws (two Woodcock flights each) a photon lane makes per warp step:
-// a warp does not wait for its lane with the longest run of virtual flights.
-#ifndef DPM_PHOTON_DRAWS
-#define DPM_PHOTON_DRAWS 1
-#endif
 constexpr int kSpillProbes = 8;
+
+// Where a warp looks for particles (see the refill loop of k_queue).
+constexpr unsigned kAskOBit = 2, kAskProbeBit = 4;
+constexpr unsigned kAskS = 1, kAskO = 1 | kAskOBit, kAskSProbe = 1 | kAskProbeBit, kAskOProbe = 1 | kAskOBit | kAskProbeBit,
+                   kAskSource = 8;
 
 struct alignas(128) Ctl {
   unsigned long long v;
   unsigned long long pad[15];
 };
 
+// A queued particle: three 16-byte words, so that a lane writes or reads its
+// record with three vector accesses.  (One array per component took twelve
+// 4-byte accesses, each with its own 64-bit address, and a sector each where
+// one or two lanes push, which is the usual case.)
+struct alignas(16) Rec {
+  float4 a;  // x, y, z, u
+  float4 b;  // v, w, E, packed voxel index
+  uint4 c;   // id low, id high, history (bit 31: positron), tag
+};
+
+// A particle's tag: the index of its history's batch, and in a shared launch
+// its job (at most 1024 batches and kSharedJobs jobs).
+constexpr int kTagJobShift = 16;
+constexpr uint32_t kTagPhoton = 0x80000000u;   // a photon in an out buffer
+constexpr uint32_t kTagPrimary = 0x40000000u;  // a source particle in a stash: its first random block is used
+
 struct QType {
-  float *x, *y, *z, *u, *v, *w, *E;
-  uint32_t *vox, *idl, *idh, *hist, *job, *seq;
+  Rec *rec;
+  uint32_t *seq;
   Ctl *head, *tail;  // [K]
 };
 
@@ -114,13 +152,14 @@ struct QDev {
   Ctl *cur_job;   // batch launches: the first job that may still have histories to
                   // start (word 0; word 1 unused)
   Ctl *job_next;  // batch launches: next history of each job [kMaxJobs]
-  int refill_min[2];  // idle lanes before a warp refills, by its particle type (photon, electron)
+  int refill_min[2];  // idle lanes before a warp takes from its stash, by its particle type (photon, electron)
+  int pause;          // steps a warp with particles waits after a fetch that found none
   uint32_t guard[2];               // per-shard bound for sources, by beam type
   long long phase_high[2], phase_low[2];  // global backlog thresholds, by beam type
   uint32_t limit;  // pushes beyond this occupancy of a shard spill over (fault injection can lower it)
   unsigned long long timeout_ns;   // bound on any single wait
   unsigned long long deadline_ns;  // bound on the whole launch (from kernel start)
-  uint64_t batch_size;
+  uint32_t batch_size;  // histories per batch (single runs)
 };
 
 __device__ __forceinline__ unsigned long long now_ns() {
@@ -145,6 +184,17 @@ __device__ __forceinline__ void st_release32(uint32_t *p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" :: "l"(p), "r"(v) : "memory");
 }
 
+// Wait until a slot's sequence word is `want`; false when the time limit runs out.
+__device__ __forceinline__ bool wait_seq(const uint32_t *seq, uint32_t want, unsigned long long timeout_ns) {
+  if (ld_acquire32(seq) == want) return true;
+  const unsigned long long t0 = now_ns();
+  while (ld_acquire32(seq) != want) {
+    if (now_ns() - t0 > timeout_ns) return false;
+    __nanosleep(32);
+  }
+  return true;
+}
+
 // Occupancy of a shard from two relaxed loads.  The loads of head and tail
 // may be observed in either order, so a concurrent consumer can make head
 // appear ahead of tail: the difference saturates at zero.
@@ -158,37 +208,69 @@ __device__ __forceinline__ unsigned lanemask_lt() {
   return m;
 }
 
-// Lane-level sink: tally with run-length coalescing, counters, and queue
-// pushes.  kMulti: a batch launch, whose particles carry their job index.
-// kCount: also count events (steps, flights, interactions, tally atomics,
-// pushes) for the run statistics; the energy counters (emitted, escaped,
-// missed) are always kept.  The event counts live in registers across the
-// whole loop and cost about 10 % of the transport rate, so runs count them
-// only on request (dpm_run_opts.count_events).  kSauter_: compile in the
-// photoelectron angle option (DPM_SAUTER); its code alone, unused, measured
-// 4-6 % slower, so only the single-run launches that ask for it carry it.
+// What a particle step of a batch job reads of its job: the phantom, the
+// history numbering and the tally.  A shared launch copies these records of all
+// its jobs into shared memory at the start (at most kSharedJobs), so that a
+// step reads them from shared memory instead of the job table.
+struct JobHot {
+  DevPhantom P;
+  uint64_t first;
+  uint32_t key0, key1;
+  unsigned long long *slabs;
+  uint32_t V;
+};
+
+// A warp's part of shared memory.
+struct WarpBox {
+  Rec stash[kStash];  // particles of the warp's own type, for its idle lanes (last in, first out)
+  Rec out[kOut];      // secondaries on their way to the queues
+  long long esc[32];  // energy that left the phantom, by lane
+  float held[32];     // numbers kept for the lanes' particles (QSink::hold)
+  long long emit, miss;            // emitted and missed energy (lane 0)
+  unsigned long long t_start;      // launch time of the warp
+  int cool;                        // steps before the warp, with particles, looks for work again
+  unsigned retry_ns;               // pause of an idle warp before it looks for work again
+  int err;
+};
+
+// energy counters (coarser quantum than the tally's, see kCounterScale)
+__device__ __forceinline__ long long fxc(float e) { return __float2ll_rn(e * kCounterScaleF); }
+
+// Lane-level sink: tally with run-length coalescing and counters.  kMulti: a
+// batch launch, whose particles carry their job index.  kCount: also count
+// events (steps, flights, interactions, tally atomics, pushes) for the run
+// statistics; the energy counters (emitted, escaped, missed) are always kept.
+// The event counts live in registers across the whole loop and cost about 10 %
+// of the transport rate, so runs count them only on request
+// (dpm_run_opts.count_events).  kSauter_: compile in the photoelectron angle
+// option (DPM_SAUTER); its code alone, unused, measured 4-6 % slower, so only
+// the single-run launches that ask for it carry it.
 template <bool kMulti, bool kCount, bool kSauter_ = false>
 struct QSink {
   static constexpr bool kSauter = kSauter_;
   const RunParams &R;
-  const QDev &Q;
-  int home;
-  unsigned long long *slab = nullptr;
+  const JobHot *sjobs;
+  WarpBox *box;
+  uint32_t tag = 0;  // of the particle in the lane
   int pend_v = -1;
   long long pend_q = 0;
-  long long cnt[C_N];
-  int err = 0;
+  long long cnt[C_N];  // event counts only (kCount)
 
-  __device__ QSink(const RunParams &r, const QDev &q, int h) : R(r), Q(q), home(h) {
+  __device__ QSink(const RunParams &r, const JobHot *sj, WarpBox *w) : R(r), sjobs(sj), box(w) {
 #pragma unroll
     for (int i = 0; i < C_N; ++i) cnt[i] = 0;
   }
   __device__ __forceinline__ static long long fx(float e) { return __float2ll_rn(e * 4294967296.0f); }
-  // energy counters (coarser quantum, see kCounterScale)
-  __device__ __forceinline__ static long long fxc(float e) { return __float2ll_rn(e * kCounterScaleF); }
   __device__ __forceinline__ void flush() {
     if (pend_v >= 0 && pend_q != 0) {
-      atomicAdd(slab + pend_v, (unsigned long long)pend_q);
+      unsigned long long *slabs = R.slabs;
+      uint32_t V = uint32_t(R.P.nx) * uint32_t(R.P.ny) * uint32_t(R.P.nz), b = tag;
+      if (kMulti) {
+        slabs = sjobs[tag >> kTagJobShift].slabs;
+        V = sjobs[tag >> kTagJobShift].V;
+        b = tag & ((1u << kTagJobShift) - 1);
+      }
+      atomicAdd(slabs + (uint64_t(b) * V + uint32_t(pend_v)), (unsigned long long)pend_q);
       if (kCount) ++cnt[C_ATOM];
     }
     pend_v = -1;
@@ -204,8 +286,10 @@ struct QSink {
       pend_q = q;
     }
   }
-  __device__ __forceinline__ void escape(float E) { cnt[C_ESC] += fxc(E); }
-  __device__ __forceinline__ void error(int e) { err |= e; }
+  __device__ __forceinline__ void escape(float E) { box->esc[threadIdx.x & 31] += fxc(E); }
+  __device__ __forceinline__ void error(int e) { atomicOr(&box->err, e); }
+  __device__ __forceinline__ void hold(float x) { box->held[threadIdx.x & 31] = x; }
+  __device__ __forceinline__ float held() const { return box->held[threadIdx.x & 31]; }
   __device__ __forceinline__ void count_step() {
     if (kCount) ++cnt[C_ESTEP];
   }
@@ -215,79 +299,79 @@ struct QSink {
   __device__ __forceinline__ void count_interaction() {
     if (kCount) ++cnt[C_GINT];
   }
-
-  // Warp-aggregated push of the lanes that are here together: one atomic on
-  // the shard's tail per queue type, then each lane writes its record and
-  // publishes its slot.
-  __device__ DPM_COLD void push(const Part &q) {
-    if (kCount) ++cnt[C_PUSH];
-    const int t = (q.type == PHOTON) ? 0 : 1;
-    const unsigned act = __activemask();
-    const unsigned mt = __ballot_sync(act, t == 1);
-    // one round per queue type; the masks are the same in every active lane
-    for (int tt = 0; tt < 2; ++tt) {
-      const unsigned mask = tt ? mt : (act & ~mt);
-      if (mask == 0 || t != tt) continue;
-      push_one(q, tt, mask);
-    }
+  // record of secondary o of p
+  __device__ __forceinline__ Rec record(const Part &p, const Emission &o) const {
+    Rec r;
+    r.a = make_float4(p.x, p.y, p.z, o.u);
+    r.b = make_float4(o.v, o.w, o.E, __uint_as_float(p.vx));
+    r.c = make_uint4(o.id_lo, o.id_hi, p.hist | (o.type == POSITRON ? 0x80000000u : 0u),
+                     tag | (o.type == PHOTON ? kTagPhoton : 0u));
+    return r;
   }
+};
 
-  __device__ void push_one(const Part &q, int t, unsigned mask) {
-    const int leader = __ffs(mask) - 1;
-    const int rank = __popc(mask & lanemask_lt());
+// 16 bytes at a time: the lane's own state stays in registers meanwhile.
+__device__ __forceinline__ void copy_rec(Rec *to, const Rec *from) {
+  to->a = from->a;
+  to->b = from->b;
+  to->c = from->c;
+}
+
+// Reserve n positions of queue t in the CTA's own shard, else in one of the next
+// ones (a full shard spills over): the shard and the first position, or -1.
+__device__ __forceinline__ int reserve(const QDev &Q, int t, int n, unsigned long long &base) {
+  const QType &Qt = Q.q[t];
+  int s = blockIdx.x % Q.K;
+#pragma unroll 1
+  for (int k = 0; k <= kSpillProbes && k < Q.K; ++k) {
+    if (occupancy(ld_volatile(&Qt.head[s].v), ld_volatile(&Qt.tail[s].v)) + n <= Q.limit) {
+      base = atomicAdd(&Qt.tail[s].v, (unsigned long long)n);
+      atomicAdd(&Q.backlog[t].v, (unsigned long long)n);
+      return s;
+    }
+    s = s + 1 == Q.K ? 0 : s + 1;
+  }
+  return -1;
+}
+
+// Queue the n records of the warp's out buffer: one atomic per 32 records on
+// the shard's tail and the backlog of each type.
+__device__ __forceinline__ void flush_out(const QDev &Q, WarpBox *w, int n) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+#pragma unroll 1
+  for (int i = lane; i - lane < n; i += 32) {
+    const bool have = i < n;
+    const int t = have && (w->out[i].c.w & kTagPhoton) ? 0 : 1;
+    const unsigned m0 = __ballot_sync(kFull, have && t == 0), m1 = __ballot_sync(kFull, have && t == 1);
+    const unsigned mask = t ? m1 : m0;
+    const int leader = (mask ? __ffs(mask) : 1) - 1;
     const QType &Qt = Q.q[t];
     unsigned long long base = 0;
     int shard = -1;
-    if ((int)(threadIdx.x & 31) == leader) {
-      // the CTA's own shard, else the next ones (a full shard spills over)
-      for (int k = 0; k <= kSpillProbes && k < Q.K; ++k) {
-        const int s = (home + k) % Q.K;
-        const unsigned long long h = ld_volatile(&Qt.head[s].v);
-        const unsigned long long tl = ld_volatile(&Qt.tail[s].v);
-        if (occupancy(h, tl) + __popc(mask) <= Q.limit) {
-          base = atomicAdd(&Qt.tail[s].v, (unsigned long long)__popc(mask));
-          atomicAdd(&Q.backlog[t].v, (unsigned long long)__popc(mask));
-          shard = s;
-          break;
+    if (have && lane == leader) shard = reserve(Q, t, __popc(mask), base);
+    base = __shfl_sync(kFull, base, leader) + __popc(mask & lanemask_lt());
+    shard = __shfl_sync(kFull, shard, leader);
+    if (have && shard < 0) shard = reserve(Q, t, 1, base);  // small queues: one by one where 32 do not fit
+    if (have) {
+      if (shard < 0) {
+        atomicOr(&w->err, ERR_OVERFLOW);
+        w->esc[lane] += fxc(w->out[i].b.z + ((w->out[i].c.z >> 31) ? 2.f * kMc2f : 0.f));
+      } else {
+        const unsigned long long pos = base;
+        const size_t idx = (size_t(shard) << Q.log2cs) + (uint32_t(pos) & Q.mask);
+        // wait for the consumer of position pos - capacity to have freed the slot
+        if (!wait_seq(Qt.seq + idx, uint32_t(pos), Q.timeout_ns)) {
+          atomicOr(&w->err, ERR_TIMEOUT);
+        } else {
+          copy_rec(Qt.rec + idx, w->out + i);
+          st_release32(Qt.seq + idx, uint32_t(pos + 1));
         }
       }
     }
-    base = __shfl_sync(mask, base, leader);
-    shard = __shfl_sync(mask, shard, leader);
-    if (shard < 0) {
-      err |= ERR_OVERFLOW;
-      cnt[C_ESC] += fxc(q.E + (q.type == POSITRON ? 2.f * kMc2f : 0.f));
-      return;
-    }
-    const unsigned long long p = base + rank;
-    const uint32_t slot = uint32_t(p) & Q.mask;
-    const size_t idx = (size_t(shard) << Q.log2cs) + slot;
-    // wait for the consumer of position p - capacity to have freed the slot
-    if (ld_acquire32(Qt.seq + idx) != uint32_t(p)) {
-      const unsigned long long t0 = now_ns();
-      while (ld_acquire32(Qt.seq + idx) != uint32_t(p)) {
-        if (now_ns() - t0 > Q.timeout_ns) {
-          err |= ERR_TIMEOUT;
-          return;
-        }
-        __nanosleep(64);
-      }
-    }
-    Qt.x[idx] = q.x;
-    Qt.y[idx] = q.y;
-    Qt.z[idx] = q.z;
-    Qt.u[idx] = q.u;
-    Qt.v[idx] = q.v;
-    Qt.w[idx] = q.w;
-    Qt.E[idx] = q.E;
-    Qt.vox[idx] = uint32_t(q.ix) | (uint32_t(q.iy) << 11) | (uint32_t(q.iz) << 22);
-    Qt.idl[idx] = q.id_lo;
-    Qt.idh[idx] = q.id_hi;
-    Qt.hist[idx] = q.hist | (q.type == POSITRON ? 0x80000000u : 0u);
-    if (kMulti) Qt.job[idx] = uint32_t(q.job);
-    st_release32(Qt.seq + idx, uint32_t(p + 1));
   }
-};
+  __syncwarp();
+}
 
 // Leader claims up to `want` queued positions of shard s with a CAS on its
 // head; returns the count (warp-uniform) and the first position.
@@ -295,6 +379,7 @@ __device__ __forceinline__ int claim(const QType &Qt, int s, int want, unsigned 
   int n = 0;
   unsigned long long b = 0;
   if ((threadIdx.x & 31) == 0) {
+#pragma unroll 1
     for (int tries = 0; tries < 32; ++tries) {
       const unsigned long long h = ld_volatile(&Qt.head[s].v);
       const unsigned long long t = ld_volatile(&Qt.tail[s].v);
@@ -314,76 +399,39 @@ __device__ __forceinline__ int claim(const QType &Qt, int s, int want, unsigned 
 
 // Read the record at position p of shard s (waiting for its publication) and
 // free the slot for the producer one lap later.
-template <bool kMulti>
-__device__ __forceinline__ bool take(const QDev &Q, int t, int s, unsigned long long p, Part &o, int &err) {
+__device__ __forceinline__ void take(const QDev &Q, int t, int s, unsigned long long p, Rec *to, int *err) {
   const QType &Qt = Q.q[t];
-  const uint32_t slot = uint32_t(p) & Q.mask;
-  const size_t idx = (size_t(s) << Q.log2cs) + slot;
-  if (ld_acquire32(Qt.seq + idx) != uint32_t(p + 1)) {
-    const unsigned long long t0 = now_ns();
-    while (ld_acquire32(Qt.seq + idx) != uint32_t(p + 1)) {
-      if (now_ns() - t0 > Q.timeout_ns) {
-        err |= ERR_TIMEOUT;
-        return false;
-      }
-      __nanosleep(32);
-    }
+  const size_t idx = (size_t(s) << Q.log2cs) + (uint32_t(p) & Q.mask);
+  if (!wait_seq(Qt.seq + idx, uint32_t(p + 1), Q.timeout_ns)) {
+    atomicOr(err, ERR_TIMEOUT);
+    // a particle without energy in its place: its first step ends it
+    to->a = to->b = make_float4(0.f, 0.f, 0.f, 0.f);
+    to->c = make_uint4(0u, 0u, 0u, 0u);
+    return;
   }
-  o.x = __ldcg(Qt.x + idx);
-  o.y = __ldcg(Qt.y + idx);
-  o.z = __ldcg(Qt.z + idx);
-  o.u = __ldcg(Qt.u + idx);
-  o.v = __ldcg(Qt.v + idx);
-  o.w = __ldcg(Qt.w + idx);
-  o.E = __ldcg(Qt.E + idx);
-  const uint32_t vx = __ldcg(Qt.vox + idx);
-  o.ix = int(vx & 0x7ffu);
-  o.iy = int((vx >> 11) & 0x7ffu);
-  o.iz = int(vx >> 22);
-  o.id_lo = __ldcg(Qt.idl + idx);
-  o.id_hi = __ldcg(Qt.idh + idx);
-  const uint32_t h = __ldcg(Qt.hist + idx);
-  o.hist = h & 0x7fffffffu;
-  o.type = t == 0 ? PHOTON : ((h >> 31) ? POSITRON : ELECTRON);
-  o.job = kMulti ? int(__ldcg(Qt.job + idx)) : 0;
-  o.ctr = 0;
+  to->a = __ldcg(&Qt.rec[idx].a);
+  to->b = __ldcg(&Qt.rec[idx].b);
+  to->c = __ldcg(&Qt.rec[idx].c);
   st_release32(Qt.seq + idx, uint32_t(p + (1ull << Q.log2cs)));
-  return true;
 }
 
-// Fill the warp's empty lanes from queue t (home shard first, then a few
-// others).  Returns the number of lanes filled (warp-uniform).
-template <bool kMulti>
-__device__ int refill_queue(const QDev &Q, int t, int home, int probes, unsigned empty, Part &p, bool &alive,
-                            int &err) {
-  const int want = __popc(empty);
-  if (want == 0) return 0;
+// Up to `want` particles of type t into the stash (home shard first, then
+// `probes` others).  Returns their number (warp-uniform).
+__device__ __forceinline__ int fetch_queue(const QDev &Q, int t, int probes, int want, WarpBox *w) {
   const int lane = threadIdx.x & 31;
   unsigned long long base;
-  int s = home;
-  int n = claim(Q.q[t], s, want, base);
-  for (int k = 1; n == 0 && k <= probes && k < Q.K; ++k) {
-    s = (home + k * 97) % Q.K;
+  int s = blockIdx.x % Q.K, n = 0;
+#pragma unroll 1
+  for (int k = 0; k <= probes && k < Q.K; ++k) {
     n = claim(Q.q[t], s, want, base);
+    if (n) break;
+    s = (s + 97) % Q.K;
   }
   if (n == 0) return 0;
   if (lane == 0) atomicAdd(&Q.backlog[t].v, (unsigned long long)(-(long long)n));
-  if (empty & (1u << lane)) {
-    const int rank = __popc(empty & lanemask_lt());
-    if (rank < n) alive = take<kMulti>(Q, t, s, base + rank, p, err);
-  }
+  if (lane < n) take(Q, t, s, base + lane, w->stash + lane, &w->err);
   return n;
 }
-
-// What a particle step of a batch job reads of its job: the phantom and the
-// history numbering.  A shared launch copies these records of all its jobs
-// into shared memory at the start (64 bytes each, at most kSharedJobs), so
-// that a step reads them from shared memory instead of the job table.
-struct JobHot {
-  DevPhantom P;
-  uint64_t first;
-  uint32_t key0, key1;
-};
 
 struct JobStepCtx {
   const DevTables &T;
@@ -392,70 +440,15 @@ struct JobStepCtx {
   uint32_t key0, key1;
 };
 
-__device__ __forceinline__ JobStepCtx job_step_ctx(const RunParams &R, const JobHot *sj, int j) {
-  return JobStepCtx{R.T, sj[j].P, sj[j].first, sj[j].key0, sj[j].key1};
+__device__ __forceinline__ JobStepCtx job_step_ctx(const RunParams &R, const JobHot *sj, uint32_t tag) {
+  const JobHot &J = sj[tag >> kTagJobShift];
+  return JobStepCtx{R.T, J.P, J.first, J.key0, J.key1};
 }
 
 // Context of a batch job for the source (the job table lives in global memory).
 __device__ __forceinline__ JobCtx job_ctx(const RunParams &R, int j) {
   const DevJob &J = R.jobs[j];
   return JobCtx{R.T, J.P, J.S, J.first, J.key0, J.key1};
-}
-
-// Start new source histories in the empty lanes: from the run's range, or
-// (batch) from the current job of the batch, job after job, so that one
-// job's phantom and tally are hot in L2 at a time.  A warp holding particles
-// of one type only starts histories of a job with that beam type.
-template <bool kMulti, bool kCount, bool kSauter>
-__device__ int refill_source(const RunParams &R, const QDev &Q, unsigned empty, Part &p, bool &alive,
-                             QSink<kMulti, kCount, kSauter> &sk, int &type) {
-  const int want = __popc(empty);
-  if (want == 0) return 0;
-  const int lane = threadIdx.x & 31;
-  unsigned long long b = ~0ull, n = 0;
-  int j = 0, jt = type;
-  if (lane == 0) {
-    if (!kMulti) {
-      n = R.n;
-      if (ld_volatile(&Q.next_hist->v) < R.n) b = atomicAdd(&Q.next_hist->v, (unsigned long long)want);
-    } else {
-      for (int tries = 0; tries <= R.n_jobs; ++tries) {
-        j = int(ld_volatile(&Q.cur_job[0].v));
-        if (j >= R.n_jobs) break;
-        jt = R.jobs[j].S.particle == 0 ? 0 : 1;
-        if (type >= 0 && jt != type) break;  // the current job has the other beam type
-        n = R.jobs[j].n;
-        if (ld_volatile(&Q.job_next[j].v) < n) {
-          b = atomicAdd(&Q.job_next[j].v, (unsigned long long)want);
-          if (b < n) break;
-        }
-        atomicCAS(&Q.cur_job[0].v, (unsigned long long)j, (unsigned long long)(j + 1));  // job exhausted
-        b = ~0ull;
-      }
-    }
-  }
-  b = __shfl_sync(kFull, b, 0);
-  n = __shfl_sync(kFull, n, 0);
-  j = __shfl_sync(kFull, j, 0);
-  jt = __shfl_sync(kFull, jt, 0);
-  if (b >= n) return 0;
-  type = jt;
-  if (empty & (1u << lane)) {
-    const unsigned long long hl = b + __popc(empty & lanemask_lt());
-    if (hl < n) {
-      bool hit;
-      if (kMulti) {
-        hit = make_primary(p, job_ctx(R, j), uint32_t(hl));
-        p.job = j;
-      } else {
-        hit = make_primary(p, R, uint32_t(hl));
-      }
-      sk.cnt[C_EMIT] += QSink<kMulti, kCount, kSauter>::fxc(p.E);
-      if (!hit) sk.cnt[C_MISS] += QSink<kMulti, kCount, kSauter>::fxc(p.E);
-      alive = hit;
-    }
-  }
-  return int(min((unsigned long long)want, n - b));
 }
 
 // Any queued particle anywhere, or histories left to start (warp-uniform).
@@ -536,168 +529,371 @@ __device__ __forceinline__ bool source_exhausted(const RunParams &R, const QDev 
   return __shfl_sync(kFull, e, 0);
 }
 
-__device__ void reduce_counters_q(const long long *cnt, int err, const RunParams &R) {
-#pragma unroll
-  for (int i = 0; i < C_N; ++i) {
-    long long v = cnt[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
-    if ((threadIdx.x & 31) == 0 && v != 0) atomicAdd(R.counters + i, (unsigned long long)v);
-  }
-  int e = err;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) e |= __shfl_down_sync(kFull, e, o);
-  if ((threadIdx.x & 31) == 0 && e) atomicOr(R.err, e);
+// A lane's state set aside in local memory while its warp starts histories.
+// The source's code needs some 50 registers; were the lane's state to live
+// through it, the compiler would keep part of that state in local memory for
+// the whole loop and store it on every step.
+struct Parked {
+  volatile uint32_t w[17];
+};
+
+__device__ __forceinline__ void park(Parked &k, const Part &p, uint32_t tag, int pend_v, long long pend_q) {
+  k.w[0] = __float_as_uint(p.x);
+  k.w[1] = __float_as_uint(p.y);
+  k.w[2] = __float_as_uint(p.z);
+  k.w[3] = __float_as_uint(p.u);
+  k.w[4] = __float_as_uint(p.v);
+  k.w[5] = __float_as_uint(p.w);
+  k.w[6] = __float_as_uint(p.E);
+  k.w[7] = p.vx;
+  k.w[8] = p.id_lo;
+  k.w[9] = p.id_hi;
+  k.w[10] = p.ctr;
+  k.w[11] = p.hist;
+  k.w[12] = uint32_t(p.type);
+  k.w[13] = tag;
+  k.w[14] = uint32_t(pend_v);
+  k.w[15] = uint32_t(pend_q);
+  k.w[16] = uint32_t(uint64_t(pend_q) >> 32);
 }
 
-// Eight resident blocks per SM caps the kernel at 64 registers per thread:
-// 32 warps per SM, the fastest of the register/occupancy trade-offs measured.
+__device__ __forceinline__ void unpark(const Parked &k, Part &p, uint32_t &tag, int &pend_v, long long &pend_q) {
+  p.x = __uint_as_float(k.w[0]);
+  p.y = __uint_as_float(k.w[1]);
+  p.z = __uint_as_float(k.w[2]);
+  p.u = __uint_as_float(k.w[3]);
+  p.v = __uint_as_float(k.w[4]);
+  p.w = __uint_as_float(k.w[5]);
+  p.E = __uint_as_float(k.w[6]);
+  p.vx = k.w[7];
+  p.id_lo = k.w[8];
+  p.id_hi = k.w[9];
+  p.ctr = k.w[10];
+  p.hist = k.w[11];
+  p.type = int(k.w[12]);
+  tag = k.w[13];
+  pend_v = int(k.w[14]);
+  const uint32_t lo = k.w[15], hi = k.w[16];
+  pend_q = (long long)((uint64_t(hi) << 32) | lo);
+}
+
+// Start up to 32 new source histories of beam type S into the (empty) stash:
+// from the run's range, or (batch) from the current job of the batch, job after
+// job, so that one job's phantom and tally are hot in L2 at a time.  All lanes
+// make a primary each, whatever their own particle is doing.  Returns the
+// number of particles in the stash, or -1 if no history was left to start.
+template <bool kMulti>
+__device__ __noinline__ int fetch_source(const RunParams &R, const QDev &Q, WarpBox *w, int S) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long b = ~0ull, n = 0;
+  int j = 0;
+  if (lane == 0) {
+    if (!kMulti) {
+      n = R.n;
+      if (ld_volatile(&Q.next_hist->v) < R.n) b = atomicAdd(&Q.next_hist->v, 32ull);
+    } else {
+#pragma unroll 1
+      for (int tries = 0; tries <= R.n_jobs; ++tries) {
+        j = int(ld_volatile(&Q.cur_job[0].v));
+        if (j >= R.n_jobs) break;
+        if ((R.jobs[j].S.particle == 0 ? 0 : 1) != S) break;  // the current job has the other beam type
+        n = R.jobs[j].n;
+        if (ld_volatile(&Q.job_next[j].v) < n) {
+          b = atomicAdd(&Q.job_next[j].v, 32ull);
+          if (b < n) break;
+        }
+        atomicCAS(&Q.cur_job[0].v, (unsigned long long)j, (unsigned long long)(j + 1));  // job exhausted
+        b = ~0ull;
+      }
+    }
+  }
+  b = __shfl_sync(kFull, b, 0);
+  n = __shfl_sync(kFull, n, 0);
+  j = __shfl_sync(kFull, j, 0);
+  if (b >= n) return -1;
+  const unsigned long long hl = b + lane;
+  bool hit = false;
+  long long e_emit = 0, e_miss = 0;
+  Part q;
+  if (hl < n) {
+    hit = kMulti ? make_primary(q, job_ctx(R, j), uint32_t(hl)) : make_primary(q, R, uint32_t(hl));
+    e_emit = fxc(q.E);
+    e_miss = hit ? 0 : e_emit;
+  }
+  const unsigned hits = __ballot_sync(kFull, hit);
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) {
+    e_emit += __shfl_down_sync(kFull, e_emit, o);
+    e_miss += __shfl_down_sync(kFull, e_miss, o);
+  }
+  if (lane == 0) {
+    w->emit += e_emit;
+    w->miss += e_miss;
+  }
+  if (hit) {
+    const uint32_t bs = kMulti ? uint32_t(R.jobs[j].batch_size) : Q.batch_size;
+    const uint32_t tag = uint32_t(hl) / bs | (kMulti ? uint32_t(j) << kTagJobShift : 0u) | kTagPrimary;
+    Rec &r = w->stash[__popc(hits & lanemask_lt())];
+    r.a = make_float4(q.x, q.y, q.z, q.u);
+    r.b = make_float4(q.v, q.w, q.E, __uint_as_float(q.vx));
+    r.c = make_uint4(q.id_lo, q.id_hi, q.hist, tag);
+  }
+  return __popc(hits);
+}
+
+// What fetch() found: particles in the stash (n may be 0 when a batch of
+// histories missed the phantom), their type, and whether the source is dry.
+struct Fetched {
+  int n, mode;
+  bool found, dry;
+};
+
+// Fill the empty stash of a warp of type `mode` (-1: no particles in its lanes)
+// with up to 32 particles, or `few` once the source is dry: near the end of a
+// launch the queued particles are spread over the warps.
+//
+// Source phase: warps start histories and track particles of the beam's type
+// while the secondaries of the other type pile up in the queues; secondary
+// phase: no history starts and warps track the queued particles in full warps.
+// Warps of the type out of phase finish their particles and turn over.  A
+// grid-wide phase keeps the SMs on one of the two code paths at a time.
+template <bool kMulti>
+__device__ __forceinline__ Fetched fetch(const RunParams &R, const QDev &Q, WarpBox *w, int mode, int few, bool dry, Part &p,
+                                 uint32_t &tag, int &pend_v, long long &pend_q) {
+  const int S = kMulti ? current_source_type(R, Q) : (R.S.particle == 0 ? 0 : 1);
+  const int O = 1 - S;
+  const int ph = grid_phase(Q, S, R.counters);
+  dry = dry || source_exhausted<kMulti>(R, Q);
+  // the places to look for work, first to last, four bits each; one loop
+  // over them keeps a single copy of the code
+  unsigned todo = 0;
+  Fetched f{0, mode, false, dry};
+  if (mode < 0)
+    todo = ph == 1 ? (kAskO | kAskOProbe << 4 | kAskS << 8 | kAskSProbe << 12)
+                   : (kAskS | kAskSource << 4 | kAskO << 8 | kAskOProbe << 12 | kAskSProbe << 16);
+  else if (mode == S)
+    todo = ph == 0 ? (kAskS | kAskSource << 4) : 0u;
+  else if (ph == 1 || dry)
+    todo = kAskOProbe;
+#pragma unroll 1
+  for (; todo != 0 && !f.found; todo >>= 4) {
+    const unsigned ask = todo & 15u;
+    if (ask == kAskSource) {
+      if (source_allowed(Q, blockIdx.x % Q.K, Q.guard[S])) {
+        Parked k;
+        park(k, p, tag, pend_v, pend_q);
+        const int k_src = fetch_source<kMulti>(R, Q, w, S);
+        f.found = k_src >= 0;
+        f.n = max(k_src, 0);
+        unpark(k, p, tag, pend_v, pend_q);
+        f.dry = !f.found;
+        if (f.found) f.mode = S;
+      }
+    } else {
+      const int t = (ask & kAskOBit) ? O : S;
+      f.n = fetch_queue(Q, t, (ask & kAskProbeBit) ? kStealProbes : 0, f.dry ? few : 32, w);
+      f.found = f.n != 0;
+      if (f.found) f.mode = t;
+    }
+  }
+  if (f.found && (threadIdx.x & 31) == 0) w->retry_ns = 32;
+  __syncwarp();
+  return f;
+}
+
+// A warp without particles waits until there is work within reach (true: look
+// again), or until the run is over or a time limit has passed (false).
+template <bool kMulti>
+__device__ __forceinline__ bool idle_wait(const RunParams &R, const QDev &Q, WarpBox *w) {
+  const int lane = threadIdx.x & 31;
+  const unsigned long long t0 = __shfl_sync(kFull, now_ns(), 0);
+  unsigned sleep_ns = 128;
+  __threadfence();
+  if (lane == 0) atomicAdd(&Q.idle->v, 1ull);
+#pragma unroll 1
+  for (;;) {
+    if (any_work_hint<kMulti>(R, Q)) {
+      // work exists but this warp found none within reach: retry after a
+      // short, growing pause instead of rescanning at once
+      if (lane == 0) atomicAdd(&Q.idle->v, ~0ull);  // -1
+      if (__shfl_sync(kFull, now_ns() - w->t_start > Q.deadline_ns, 0)) {
+        if (lane == 0) atomicOr(&w->err, ERR_TIMEOUT);
+        return false;
+      }
+      const unsigned ns = w->retry_ns;
+      __syncwarp();
+      __nanosleep(ns);
+      if (lane == 0) w->retry_ns = min(ns * 2, 2048u);
+      __syncwarp();
+      return true;
+    }
+    bool done = false;
+    if (lane == 0) done = ld_volatile(&Q.idle->v) == ld_volatile(&Q.started->v);
+    done = __shfl_sync(kFull, done, 0);
+    if (done) {
+      __threadfence();
+      if (!any_work<kMulti>(R, Q)) return false;
+    }
+    if (__shfl_sync(kFull, now_ns() - t0 > Q.timeout_ns, 0)) {
+      if (lane == 0) atomicOr(&w->err, ERR_TIMEOUT);
+      return false;
+    }
+    __nanosleep(sleep_ns);
+    sleep_ns = min(sleep_ns * 2, 16384u);
+  }
+}
+
+__device__ void reduce_counters_q(const long long *cnt, const WarpBox *w, const RunParams &R) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < C_N; ++i) {
+    long long v = i == C_ESC ? w->esc[lane] : i == C_EMIT ? (lane == 0 ? w->emit : 0) : i == C_MISS ? (lane == 0 ? w->miss : 0) : cnt[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
+    if (lane == 0 && v != 0) atomicAdd(R.counters + i, (unsigned long long)v);
+  }
+  if (lane == 0 && w->err) atomicOr(R.err, w->err);
+}
+
+// Six resident blocks per SM: 24 warps with 80 registers each.  At 8 (64
+// registers) and 7 (72) parts of the particle's state live in local memory in
+// the hot loop (20 MeV electrons on the slabs: 683 and 476 M L2 sectors instead
+// of 309 M), 5 (96) are as fast on short launches and 7 % slower on long ones.
 #ifndef DPM_QUEUE_MIN_BLOCKS
-#define DPM_QUEUE_MIN_BLOCKS 8
+#define DPM_QUEUE_MIN_BLOCKS 6
 #endif
-template <bool kMulti, bool kCount, bool kSauter = false, bool kPause = false>
+template <bool kMulti, bool kCount, bool kSauter = false>
 __global__ void __launch_bounds__(kQBlock, DPM_QUEUE_MIN_BLOCKS)
     k_queue(const __grid_constant__ RunParams R, const __grid_constant__ QDev Q) {
+  __shared__ WarpBox s_box[kQBlock / 32];
+  extern __shared__ JobHot sjobs[];
   const int lane = threadIdx.x & 31;
-  const int home = blockIdx.x % Q.K;
-  const int src_type = (R.S.particle == 0) ? 0 : 1;
-  const size_t V = size_t(R.P.nx) * R.P.ny * R.P.nz;
-  if (lane == 0) atomicAdd(&Q.started->v, 1ull);
-  QSink<kMulti, kCount, kSauter> sk(R, Q, home);
-  Part p{};
-  bool alive = false;
-  int nstep = 0;
-  int mode = -1;  // warp-uniform: type of the particles in the lanes, -1 when empty
-  bool idle = false;
-  unsigned long long idle_t0 = 0;
-  unsigned sleep_ns = 128;
-  unsigned retry_ns = 32;
-  const unsigned long long t_start = __shfl_sync(kFull, now_ns(), 0);
+  WarpBox *box = s_box + (threadIdx.x >> 5);
+  box->esc[lane] = 0;
+  if (lane == 0) {
+    box->emit = box->miss = 0;
+    box->t_start = now_ns();
+    box->retry_ns = 32;
+    box->cool = 0;
+    box->err = 0;
+    atomicAdd(&Q.started->v, 1ull);
+  }
   // batch launches: the jobs' step records in shared memory (all threads of
   // the block are here, before any divergent code)
-  extern __shared__ JobHot sjobs[];
   if (kMulti) {
     for (int j = threadIdx.x; j < R.n_jobs; j += blockDim.x) {
       const DevJob &J = R.jobs[j];
-      sjobs[j] = JobHot{J.P, J.first, J.key0, J.key1};
+      sjobs[j] = JobHot{J.P, J.first, J.key0, J.key1, J.slabs, uint32_t(J.V)};
     }
-    __syncthreads();
   }
-  int cool = 0;  // warp-uniform (kPause): steps before a warp with particles tries to refill again
+  __syncthreads();
+  QSink<kMulti, kCount, kSauter> sk(R, sjobs, box);
+  Part p{};
+  bool alive = false;
+  // warp-uniform from here on
+  int n_stash = 0, n_out = 0;  // records in the stash (all of type `mode`) and in the out buffer
+  int mode = -1;               // type of the particles in the lanes, -1 without any
+  bool dry = false;            // the source had nothing left when last asked
   for (;;) {
-    unsigned live = __ballot_sync(kFull, alive);
-    if (live == 0) mode = -1;
-    const unsigned live_before = live;
-    if (kPause && live != 0 && cool > 0) {
-      --cool;
-    } else if (live == 0 || 32 - __popc(live) >= Q.refill_min[mode > 0 ? 1 : 0]) {
-      const unsigned empty = ~live;
-      const bool was_alive = alive;
-      const int S = kMulti ? current_source_type(R, Q) : src_type;
-      // Source phase: warps start histories and track particles of the
-      // beam's type while the secondaries of the other type pile up in
-      // the queues; secondary phase: no history starts and warps track the
-      // queued particles in full warps.  Warps of the type out of phase
-      // finish their lanes and turn over.  A grid-wide phase keeps the SMs
-      // on one of the two code paths at a time.
-      const int O = 1 - S;
-      const int ph = grid_phase(Q, S, R.counters);
-      if (mode < 0) {
-        if (ph == 1) {
-          if (refill_queue<kMulti>(Q, O, home, 0, empty, p, alive, sk.err)) mode = O;
-          else if (refill_queue<kMulti>(Q, O, home, kStealProbes, empty, p, alive, sk.err)) mode = O;
-          else if (refill_queue<kMulti>(Q, S, home, 0, empty, p, alive, sk.err)) mode = S;
-          else if (refill_queue<kMulti>(Q, S, home, kStealProbes, empty, p, alive, sk.err)) mode = S;
-        } else {
-          int ty = S;
-          if (refill_queue<kMulti>(Q, S, home, 0, empty, p, alive, sk.err)) mode = S;
-          else if (source_allowed(Q, home, Q.guard[S]) && refill_source<kMulti, kCount, kSauter>(R, Q, empty, p, alive, sk, ty)) mode = S;
-          else if (refill_queue<kMulti>(Q, O, home, 0, empty, p, alive, sk.err)) mode = O;
-          else if (refill_queue<kMulti>(Q, O, home, kStealProbes, empty, p, alive, sk.err)) mode = O;
-          else if (refill_queue<kMulti>(Q, S, home, kStealProbes, empty, p, alive, sk.err)) mode = S;
-        }
-      } else if (mode == S) {
-        int ty = S;
-        if (ph == 0 && !refill_queue<kMulti>(Q, S, home, 0, empty, p, alive, sk.err) && source_allowed(Q, home, Q.guard[S]))
-          refill_source<kMulti, kCount, kSauter>(R, Q, empty, p, alive, sk, ty);
-      } else if (ph == 1 || source_exhausted<kMulti>(R, Q)) {
-        refill_queue<kMulti>(Q, O, home, kStealProbes, empty, p, alive, sk.err);
-      }
-      if (alive && !was_alive) {
-        if (kMulti) {
-          const DevJob &J = R.jobs[p.job];
-          sk.slab = J.slabs + (uint64_t(p.hist) / J.batch_size) * J.V;
-        } else {
-          sk.slab = R.slabs + (uint64_t(p.hist) / Q.batch_size) * V;
-        }
-        nstep = 0;
-      }
-      live = __ballot_sync(kFull, alive);
-      if (live != 0u) {
-        retry_ns = 32;
-        sleep_ns = 128;
-      }
-      if (kPause) cool = (live != 0u && live == live_before) ? DPM_REFILL_COOLDOWN : 0;
+    const unsigned live = __ballot_sync(kFull, alive);
+    const int n_idle = 32 - __popc(live);
+    // near the end of a launch every particle is for whoever is idle
+    const bool send = n_out > kOut - 32 || (n_out != 0 && (dry || live == 0));
+    bool look = live == 0 && n_stash == 0;
+    if (live == 0 && n_stash == 0) {
+      mode = -1;
+    } else if (n_stash == 0 && n_idle >= DPM_FETCH_MIN) {
+      const int c = box->cool;
+      __syncwarp();
+      if (lane == 0 && c > 0) box->cool = c - 1;
+      look = c == 0;
     }
-    if (live == 0) {
-      // nothing in the lanes: idle until work appears or the run is over
-      if (!idle) {
-        __threadfence();
-        if (lane == 0) atomicAdd(&Q.idle->v, 1ull);
-        idle = true;
-        idle_t0 = now_ns();
-      }
-      if (any_work_hint<kMulti>(R, Q)) {
-        // work exists but this warp found none within reach: retry after a
-        // short, growing pause instead of rescanning at once
-        if (lane == 0) atomicAdd(&Q.idle->v, ~0ull);  // -1
-        idle = false;
-        if (__shfl_sync(kFull, now_ns() - t_start > Q.deadline_ns, 0)) {
-          sk.error(ERR_TIMEOUT);
-          break;
+    if (send) {
+      flush_out(Q, box, n_out);
+      n_out = 0;
+    }
+    if (look) {
+      const Fetched f = fetch<kMulti>(R, Q, box, mode, n_idle, dry, p, sk.tag, sk.pend_v, sk.pend_q);
+      n_stash = f.n;
+      mode = f.mode;
+      dry = f.dry;
+      if (lane == 0) box->cool = f.found ? 0 : Q.pause;
+      __syncwarp();
+    }
+    if (n_idle >= Q.refill_min[mode > 0 ? 1 : 0] || live == 0) {
+      if (n_stash != 0) {
+        // the newest records into the idle lanes
+        __syncwarp();
+        const int rank = __popc(~live & lanemask_lt());
+        if (!alive && rank < n_stash) {
+          const Rec &r = box->stash[n_stash - 1 - rank];
+          const float4 a = r.a, b = r.b;
+          const uint4 c = r.c;
+          p.x = a.x;
+          p.y = a.y;
+          p.z = a.z;
+          p.u = a.w;
+          p.v = b.x;
+          p.w = b.y;
+          p.E = b.z;
+          p.vx = __float_as_uint(b.w);
+          p.id_lo = c.x;
+          p.id_hi = c.y;
+          p.hist = c.z & 0x7fffffffu;
+          p.type = mode == 0 ? PHOTON : (c.z >> 31) ? POSITRON : ELECTRON;
+          p.ctr = (c.w & kTagPrimary) ? 1u : 0u;
+          sk.tag = c.w & ~(kTagPhoton | kTagPrimary);
+          alive = true;
         }
-        __nanosleep(retry_ns);
-        retry_ns = min(retry_ns * 2, 2048u);
+        __syncwarp();
+        n_stash = max(n_stash - n_idle, 0);
+      } else if (live == 0) {
+        if (!idle_wait<kMulti>(R, Q, box)) break;
+        p = Part{};  // nothing in the lanes: no state to keep through the wait
+        sk.tag = 0;
+        sk.pend_v = -1;
+        sk.pend_q = 0;
         continue;
       }
-      bool done = false;
-      if (lane == 0) done = ld_volatile(&Q.idle->v) == ld_volatile(&Q.started->v);
-      done = __shfl_sync(kFull, done, 0);
-      if (done) {
-        __threadfence();
-        if (!any_work<kMulti>(R, Q)) break;
-      }
-      const bool expired = __shfl_sync(kFull, now_ns() - idle_t0 > Q.timeout_ns, 0);
-      if (expired) {
-        sk.error(ERR_TIMEOUT);
-        break;
-      }
-      __nanosleep(sleep_ns);
-      sleep_ns = min(sleep_ns * 2, 16384u);
-      continue;
     }
+    const bool was = alive;
+    Emission o;
     if (alive) {
-      if (mode == 0) {
-        alive = kMulti ? photon_segment(p, job_step_ctx(R, sjobs, p.job), sk, DPM_PHOTON_DRAWS)
-                       : photon_segment(p, R, sk, DPM_PHOTON_DRAWS);
-        if (alive && ++nstep >= kMaxPhotonSegments * 8) {
-          sk.error(ERR_STEPCAP);
-          sk.deposit(kMulti ? vox(p, sjobs[p.job].P) : vox(p, R.P), p.E);
-          alive = false;
-        }
-      } else {
-        alive = kMulti ? electron_step(p, job_step_ctx(R, sjobs, p.job), sk) : electron_step(p, R, sk);
-        if (alive && ++nstep >= kMaxElectronSteps) {
-          sk.error(ERR_STEPCAP);
-          sk.deposit(kMulti ? vox(p, sjobs[p.job].P) : vox(p, R.P), p.E);
-          alive = false;
-        }
+      if (p.type & CHAIN)
+        alive = kMulti ? chain_step(p, job_step_ctx(R, sjobs, sk.tag), sk, o) : chain_step(p, R, sk, o);
+      else if (mode == 0)
+        alive = kMulti ? photon_flight(p, job_step_ctx(R, sjobs, sk.tag), sk, o) : photon_flight(p, R, sk, o);
+      else
+        alive = kMulti ? electron_step(p, job_step_ctx(R, sjobs, sk.tag), sk, o) : electron_step(p, R, sk, o);
+      if (alive && p.ctr >= (mode == 0 ? kMaxPhotonBlocks : kMaxElectronBlocks)) {
+        sk.error(ERR_STEPCAP);
+        sk.deposit(kMulti ? vox(p, job_step_ctx(R, sjobs, sk.tag).P) : vox(p, R.P), p.E);
+        alive = false;
       }
-      if (!alive) sk.flush();
+    }
+    // The step's secondaries, in one place for the whole warp whatever made
+    // them: those of the warp's own type go to its stash while it has room,
+    // the others to the queues by way of the out buffer (which has room for 32).
+    bool want = false;
+    if (o.kind != EM_NONE) want = kMulti ? settle(p, o, job_step_ctx(R, sjobs, sk.tag), sk) : settle(p, o, R, sk);
+    if (was && !alive) sk.flush();
+    const unsigned all = __ballot_sync(kFull, want);
+    if (all != 0) {
+      if (kCount && want) ++sk.cnt[C_PUSH];
+      const unsigned own = __ballot_sync(kFull, want && (o.type == PHOTON) == (mode == 0));
+      const bool keep = !dry && n_stash + __popc(own) <= kStash;
+      const unsigned to_out = keep ? all & ~own : all;
+      if (want) {
+        const bool st = keep && (own >> lane & 1u);
+        Rec *dst = st ? box->stash + n_stash + __popc(own & lanemask_lt()) : box->out + n_out + __popc(to_out & lanemask_lt());
+        *dst = sk.record(p, o);
+      }
+      if (keep) n_stash += __popc(own);
+      n_out += __popc(to_out);
     }
   }
-  sk.flush();
-  reduce_counters_q(sk.cnt, sk.err, R);
+  __syncwarp();
+  reduce_counters_q(sk.cnt, box, R);
 }
 
 __global__ void k_queue_init(uint32_t *seq0, uint32_t *seq1, size_t n, uint32_t mask) {
@@ -710,47 +906,33 @@ __global__ void k_queue_init(uint32_t *seq0, uint32_t *seq1, size_t n, uint32_t 
 }  // namespace
 
 // The queue kernel's instantiations: single run or batch launch (kMulti) x
-// event counts x refill pause, and the single runs with the photoelectron
-// angle option.
+// event counts, and the single runs with the photoelectron angle option.
 using QKernel = void (*)(RunParams, QDev);
 struct QKernelEntry {
   QKernel k;
   bool multi;
 };
-const QKernelEntry kQueueKernels[10] = {
-    {k_queue<false, false>, false},
-    {k_queue<false, true>, false},
-    {k_queue<true, false>, true},
-    {k_queue<true, true>, true},
-    {k_queue<false, false, true>, false},
-    {k_queue<false, true, true>, false},
-    {k_queue<false, false, false, true>, false},
-    {k_queue<false, true, false, true>, false},
-    {k_queue<true, false, false, true>, true},
-    {k_queue<true, true, false, true>, true}};
+const QKernelEntry kQueueKernels[6] = {
+    {k_queue<false, false>, false},      {k_queue<false, true>, false},      {k_queue<true, false>, true},
+    {k_queue<true, true>, true},         {k_queue<false, false, true>, false}, {k_queue<false, true, true>, false}};
 
-QKernel queue_kernel(bool multi, bool count, bool sauter, bool pause) {
+QKernel queue_kernel(bool multi, bool count, bool sauter) {
   if (sauter) return count ? k_queue<false, true, true> : k_queue<false, false, true>;
-  if (multi) {
-    if (pause) return count ? k_queue<true, true, false, true> : k_queue<true, false, false, true>;
-    return count ? k_queue<true, true> : k_queue<true, false>;
-  }
-  if (pause) return count ? k_queue<false, true, false, true> : k_queue<false, false, false, true>;
+  if (multi) return count ? k_queue<true, true> : k_queue<true, false>;
   return count ? k_queue<false, true> : k_queue<false, false>;
 }
 
 int queue_blocks_per_sm() {
-  // single runs keep no shared memory: the whole carveout goes to L1, where
-  // the tables are cached; a batch launch keeps its jobs' step records there
-  // (kSharedJobs x 64 bytes per block: 8 blocks with their reserved 1 KB
-  // each need the 64 KB configuration, 28 % of the 228 KB)
+  // Shared memory for the resident blocks (17 KB of stashes and buffers each,
+  // in a batch launch also the step records of up to kSharedJobs jobs, and 1 KB
+  // reserved), the rest to L1, where the tables are cached.
   int best = 1 << 30;
   for (const QKernelEntry &e : kQueueKernels) {
     const QKernel k = e.k;
     int per_sm = 0;
     const bool multi = e.multi;
     const size_t smem = multi ? kSharedJobs * sizeof(JobHot) : 0;
-    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, multi ? 28 : 0);
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, multi ? 64 : 50);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kQBlock, smem) != cudaSuccess) {
       cudaGetLastError();
       return 0;
@@ -772,7 +954,8 @@ int queue_preload() {
   return queue_blocks_per_sm();
 }
 
-constexpr int kWordsPerSlot = 13;  // x y z u v w E, voxel, id lo, id hi, history, job, sequence
+constexpr int kWordsPerSlot = 13;  // a record and its sequence word
+static_assert(sizeof(Rec) + 4 == kWordsPerSlot * 4, "record layout");
 constexpr int kCtlWords = 8 + kMaxJobs;  // next_hist idle started cur_job[2] backlog[2] phase, job_next[kMaxJobs]
 
 size_t queue_bytes(int K, int log2cs) {
@@ -809,15 +992,8 @@ int queue_launch(void *mem, int K, int log2cs, const RunParams &R, uint64_t batc
     char *b = ctl_end + t * per_type;
     T.head = reinterpret_cast<Ctl *>(b);
     T.tail = T.head + K;
-    uint32_t *f = reinterpret_cast<uint32_t *>(b + 2 * size_t(K) * sizeof(Ctl));
-    float **fl[7] = {&T.x, &T.y, &T.z, &T.u, &T.v, &T.w, &T.E};
-    for (int i = 0; i < 7; ++i) *fl[i] = reinterpret_cast<float *>(f + i * slots);
-    T.vox = f + 7 * slots;
-    T.idl = f + 8 * slots;
-    T.idh = f + 9 * slots;
-    T.hist = f + 10 * slots;
-    T.job = f + 11 * slots;
-    T.seq = f + 12 * slots;
+    T.rec = reinterpret_cast<Rec *>(b + 2 * size_t(K) * sizeof(Ctl));
+    T.seq = reinterpret_cast<uint32_t *>(T.rec + slots);
   }
   Q.K = K;
   Q.log2cs = log2cs;
@@ -837,7 +1013,7 @@ int queue_launch(void *mem, int K, int log2cs, const RunParams &R, uint64_t batc
   // the whole launch: the wait bound plus 2 us per history (a hundred times the
   // cost of a 20 MeV electron history on this path)
   Q.deadline_ns = Q.timeout_ns + (unsigned long long)(double(R.n) * 2000.0);
-  Q.batch_size = batch_size;
+  Q.batch_size = uint32_t(batch_size);
   // zero the control words of both types and the run counters
   const int n_ctl = R.jobs ? 8 + R.n_jobs : 8;
   cudaError_t e = cudaMemsetAsync(m, 0, n_ctl * sizeof(Ctl), st);
@@ -850,15 +1026,10 @@ int queue_launch(void *mem, int K, int log2cs, const RunParams &R, uint64_t batc
   if (start) cudaEventRecord(start, st);
   const bool count = o.count_events != 0;
   const bool sauter = (R.T.flags & DPM_SAUTER) != 0;
-  bool pause = o.refill_pause > 0;
-  if (o.refill_pause == 0) {
-    // single run: from its own histories (callers on queues below
-    // 2^kPauseMinLog2 slots pass -1); a batch launch's caller decides
-    const double w = R.S.particle == 0 ? 1.0 : kElectronHistoryWeight;
-    pause = !R.jobs && double(R.n) * w <= kPauseMaxHistories;
-  }
+  const bool pause = o.refill_pause >= 0;  // callers on queues below 2^kPauseMinLog2 slots pass -1 for 0
+  Q.pause = pause ? DPM_REFILL_COOLDOWN : 0;
   const size_t smem = R.jobs ? size_t(R.n_jobs) * sizeof(JobHot) : 0;
-  queue_kernel(R.jobs != nullptr, count, sauter, pause)<<<K, kQBlock, smem, st>>>(R, Q);
+  queue_kernel(R.jobs != nullptr, count, sauter)<<<K, kQBlock, smem, st>>>(R, Q);
   e = cudaGetLastError();
   if (e != cudaSuccess) {
     err = cudaGetErrorString(e);

@@ -32,16 +32,9 @@ int queue_prepare(QueueState &q, const dpm_run_opts &o, int sm_count, int &K, in
 constexpr int kSharedJobs = 64;
 
 // A launch pauses refills that found nothing (dpm_run_opts.refill_pause = 0)
-// when its work is at most kPauseMaxHistories 6 MV photon histories, an
-// electron-beam history counting kElectronHistoryWeight (20 MeV electrons run
-// at about an eighth of the 6 MV beam's histories/s).  The pause shortens the
-// end of a launch by about 0.3 ms and costs about 1.5 % in between, so it
-// pays below about 2x10^7 photon histories.
-constexpr double kPauseMaxHistories = 1.6e7;
-constexpr double kElectronHistoryWeight = 8.0;
-// ... and only with shards of at least 2^kPauseMinLog2 slots: small queues
-// (the no-allocation entry point's, or a small queue_log2) need every refill
-// to keep the producers' shards from overflowing.
+// with shards of at least 2^kPauseMinLog2 slots: small queues (the
+// no-allocation entry point's, or a small queue_log2) need every refill to keep
+// the producers' shards from overflowing.
 constexpr int kPauseMinLog2 = 13;
 
 // Resident blocks per SM of the queue kernel (occupancy query), or 0 on error.
