@@ -60,11 +60,11 @@ int batch_device_work(dpm_ctx *c, const Prepared &b, const RunParams &R, const d
       return ctx_fail(c, rc, err);
   for (size_t j = 0; j < b.tab.size(); ++j) {
     PhantomState *p = b.ph[j];
-    launch_fold(p->d_slabs, b.nb[j], p->V, p->d_inv_nb, p->d_S1, p->d_Q, c->sm_count, c->stream);
+    ctx_fold(c, p, b.tab[j].n, b.tab[j].batch_size, b.nb[j]);
   }
   for (size_t j = 0; j < b.solo.size(); ++j) {
     PhantomState *p = b.solo_ph[j];
-    launch_fold(p->d_slabs, b.solo_nb[j], p->V, p->d_inv_nb, p->d_S1, p->d_Q, c->sm_count, c->stream);
+    ctx_fold(c, p, b.solo[j].n, b.solo_bs[j], b.solo_nb[j]);
   }
   BATCH_TRY(c, cudaGetLastError());
   return DPM_OK;

@@ -96,7 +96,7 @@ void free_phantom(dpm_ctx *c, PhantomState *p) {
   drop_events(p);
   for (void *d : {(void *)p->d_mat, (void *)p->d_rho, (void *)p->d_mumax, (void *)p->d_mumax64, (void *)p->d_slabs,
                   (void *)p->d_fslabs,
-                  (void *)p->d_S1, (void *)p->d_Q, (void *)p->d_counters, (void *)p->d_inv_nb, (void *)p->d_dose,
+                  (void *)p->d_S1, (void *)p->d_Q, (void *)p->d_counters, (void *)p->d_dose,
                   (void *)p->d_sigma, (void *)p->d_dmax})
     dfree(c, d);
 }
@@ -189,11 +189,12 @@ int ctx_prepare_batches(dpm_ctx *c, PhantomState *p, uint64_t n, int n_batches, 
     if ((rc = dalloc(c, &p->d_slabs, size_t(B) * p->V))) return rc;
     p->slab_batches = size_t(B);
   }
-  std::vector<double> inv_nb(B);
-  for (int b = 0; b < B; ++b) inv_nb[b] = 1.0 / double(std::min<uint64_t>(bs, n - uint64_t(b) * bs));
-  CUDA_TRY(c, cudaMemcpyAsync(p->d_inv_nb, inv_nb.data(), B * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  // pageable source: the copy is staged before the call returns
   return DPM_OK;
+}
+
+void ctx_fold(dpm_ctx *c, PhantomState *p, uint64_t n, uint64_t bs, int B) {
+  launch_fold(p->d_slabs, B, p->V, 1.0 / double(std::min(bs, n)), 1.0 / double(n - uint64_t(B - 1) * bs), p->d_S1, p->d_Q,
+              c->sm_count, c->stream);
 }
 
 PhantomState *ctx_phantom(dpm_ctx *c, int id) { return get_phantom(c, id); }
@@ -420,8 +421,8 @@ int dpm_load_phantom(dpm_ctx *c, int nx, int ny, int nz, double dx, double dy, d
   int rc;
   if ((rc = scan_phantom(c, mat, rho, p->V, p->max_mat, p->rho_max))) return rc;
   if ((rc = dalloc(c, &p->d_mat, p->V)) || (rc = dalloc(c, &p->d_rho, p->V)) || (rc = dalloc(c, &p->d_S1, p->V)) ||
-      (rc = dalloc(c, &p->d_Q, p->V)) || (rc = dalloc(c, &p->d_counters, size_t(kCounterSlots))) ||
-      (rc = dalloc(c, &p->d_inv_nb, size_t(1024))) || (rc = dalloc(c, &p->d_mumax, size_t(kMaxTableNodes)))) {
+      (rc = dalloc(c, &p->d_Q, p->V)) || (rc = dalloc(c, &p->d_counters, size_t(kCounterSlots + kSumSlots))) ||
+      (rc = dalloc(c, &p->d_mumax, size_t(kMaxTableNodes)))) {
     free_phantom(c, p.get());
     return rc;
   }
@@ -584,8 +585,8 @@ int dpm_clone_phantom(dpm_ctx *c, int src_id, int *phantom_id) {
   for (int m = 0; m < DPM_MAX_MAT; ++m) p->rho_max[m] = s->rho_max[m];
   int rc;
   if ((rc = dalloc(c, &p->d_mat, p->V)) || (rc = dalloc(c, &p->d_rho, p->V)) || (rc = dalloc(c, &p->d_S1, p->V)) ||
-      (rc = dalloc(c, &p->d_Q, p->V)) || (rc = dalloc(c, &p->d_counters, size_t(kCounterSlots))) ||
-      (rc = dalloc(c, &p->d_inv_nb, size_t(1024))) || (rc = dalloc(c, &p->d_mumax, size_t(kMaxTableNodes)))) {
+      (rc = dalloc(c, &p->d_Q, p->V)) || (rc = dalloc(c, &p->d_counters, size_t(kCounterSlots + kSumSlots))) ||
+      (rc = dalloc(c, &p->d_mumax, size_t(kMaxTableNodes)))) {
     free_phantom(c, p.get());
     return rc;
   }
@@ -705,7 +706,7 @@ int dpm_run(dpm_ctx *c, int id, const dpm_source *src, uint64_t first, uint64_t 
   }
   CUDA_TRY(c, cudaGetLastError());
   CUDA_TRY(c, cudaEventRecord(ev[1], c->stream));
-  launch_fold(p->d_slabs, B, p->V, p->d_inv_nb, p->d_S1, p->d_Q, c->sm_count, c->stream);
+  ctx_fold(c, p, n, bs, B);
   CUDA_TRY(c, cudaGetLastError());
   CUDA_TRY(c, cudaEventRecord(ev[2], c->stream));
   p->n_total += n;
@@ -735,32 +736,23 @@ int dpm_sync(dpm_ctx *c) {
   return DPM_OK;
 }
 
-// Fill the run summary; s1_host (if not NULL) already holds the integer tally.
-static int read_common(dpm_ctx *c, PhantomState *p, const int64_t *s1_host, dpm_run_stats *st, int sync_rc) {
+// Queue the sum of the tally, which fill_stats() reads.
+static void queue_sums(dpm_ctx *c, PhantomState *p) {
+  launch_sum_tally(p->d_S1, p->V, p->d_counters + kCounterSlots, c->sm_count, c->stream);
+}
+
+// Fill the run summary (after queue_sums() and a wait for the stream).
+static int fill_stats(dpm_ctx *c, PhantomState *p, dpm_run_stats *st, int sync_rc) {
   if (st) {
-    unsigned long long cnt[kCounterSlots];
+    unsigned long long cnt[kCounterSlots + kSumSlots];
     CUDA_TRY(c, cudaMemcpy(cnt, p->d_counters, sizeof(cnt), cudaMemcpyDeviceToHost));
     std::memset(st, 0, sizeof(*st));
     st->n_histories = p->n_total;
     st->n_batches = int32_t(p->b_total);
-    // the voxel sum can exceed an int64 of 2^-32 MeV quanta: summed exactly,
-    // the high (signed) and low 32-bit halves apart, neither of which can
-    // overflow 64 bits below 2^32 voxels (the largest phantom has fewer), then
+    // the voxel sum can exceed an int64 of 2^-32 MeV quanta: summed exactly, then
     // rounded once
-    std::vector<long long> s1;
-    const int64_t *src = s1_host;
-    if (!src) {
-      s1.resize(p->V);
-      CUDA_TRY(c, cudaMemcpy(s1.data(), p->d_S1, p->V * sizeof(long long), cudaMemcpyDeviceToHost));
-      src = reinterpret_cast<const int64_t *>(s1.data());
-    }
-    int64_t hi = 0;
-    uint64_t lo = 0;
-    for (size_t v = 0; v < p->V; ++v) {
-      hi += src[v] >> 32;  // arithmetic shift: floor(x / 2^32)
-      lo += uint64_t(src[v]) & 0xffffffffull;
-    }
-    const __int128 dep = (__int128)hi * 4294967296 + (__int128)lo;
+    const __int128 dep =
+        (__int128)(long long)cnt[kCounterSlots] * 4294967296 + (__int128)cnt[kCounterSlots + 1];
     st->emitted = double((long long)cnt[C_EMIT]) / kCounterScale;
     st->escaped = double((long long)cnt[C_ESC]) / kCounterScale;
     st->missed = double((long long)cnt[C_MISS]) / kCounterScale;
@@ -794,24 +786,22 @@ int dpm_read_dose(dpm_ctx *c, int id, double *dose, double *sigma, int64_t *s1_r
   if (!c) return DPM_EINVAL;
   PhantomState *p = get_phantom(c, id);
   if (!p) return fail(c, DPM_EINVAL, "bad phantom id");
-  const int src = dpm_sync(c);
-  if (src == DPM_ECUDA) return src;
-  std::string keep = c->err;
+  cudaSetDevice(c->device);
   if (dose || sigma) {
     int rc;
     if (!p->d_dose && ((rc = dalloc(c, &p->d_dose, p->V)) || (rc = dalloc(c, &p->d_sigma, p->V)))) return rc;
     launch_normalize(p->d_S1, p->d_Q, p->d_rho, p->V, double(p->n_total), double(p->b_total), p->dx * p->dy * p->dz,
                      p->d_dose, p->d_sigma, c->sm_count, c->stream);
-    CUDA_TRY(c, cudaGetLastError());
-    if (dose) CUDA_TRY(c, cudaMemcpyAsync(dose, p->d_dose, p->V * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    if (sigma) CUDA_TRY(c, cudaMemcpyAsync(sigma, p->d_sigma, p->V * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   }
+  if (st) queue_sums(c, p);
+  CUDA_TRY(c, cudaGetLastError());
+  if (dose) CUDA_TRY(c, cudaMemcpyAsync(dose, p->d_dose, p->V * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  if (sigma) CUDA_TRY(c, cudaMemcpyAsync(sigma, p->d_sigma, p->V * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   if (s1_raw) CUDA_TRY(c, cudaMemcpyAsync(s1_raw, p->d_S1, p->V * sizeof(long long), cudaMemcpyDeviceToHost, c->stream));
-  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  int rc = read_common(c, p, s1_raw, st, src);
-  if (rc) return rc;
-  if (src) c->err = keep;
-  return src;
+  const int src = dpm_sync(c);
+  if (src == DPM_ECUDA) return src;
+  const int rc = fill_stats(c, p, st, src);
+  return rc ? rc : src;
 }
 
 int dpm_read_dose_device(dpm_ctx *c, int id, double *d_dose, double *d_sigma, dpm_run_stats *st) {
@@ -821,15 +811,13 @@ int dpm_read_dose_device(dpm_ctx *c, int id, double *d_dose, double *d_sigma, dp
   cudaSetDevice(c->device);
   launch_normalize(p->d_S1, p->d_Q, p->d_rho, p->V, double(p->n_total), double(p->b_total), p->dx * p->dy * p->dz,
                    d_dose, d_sigma, c->sm_count, c->stream);
+  if (st) queue_sums(c, p);
   CUDA_TRY(c, cudaGetLastError());
   if (!st) return DPM_OK;
   const int src = dpm_sync(c);
   if (src == DPM_ECUDA) return src;
-  std::string keep = c->err;
-  int rc = read_common(c, p, nullptr, st, src);
-  if (rc) return rc;
-  if (src) c->err = keep;
-  return src;
+  const int rc = fill_stats(c, p, st, src);
+  return rc ? rc : src;
 }
 
 // ---------------------------------------------------------------------------

@@ -42,7 +42,6 @@ struct PhantomState {
   long long *d_S1 = nullptr;
   double *d_Q = nullptr;
   unsigned long long *d_counters = nullptr;
-  double *d_inv_nb = nullptr;
   double *d_dose = nullptr, *d_sigma = nullptr;
   unsigned long long *d_dmax = nullptr;  // [1] key + [3] doubles for the D_max query
   uint64_t n_total = 0;
@@ -110,9 +109,11 @@ int ctx_run_params_f64(dpm_ctx *c, PhantomState *p, const dpm_source *src, uint6
                        uint64_t seed, int physics_flags, RunParamsT<double> &R);
 // Device allocation owned by the context (error message set on failure).
 int ctx_alloc(dpm_ctx *c, void **p, size_t bytes);
-// Batch structure of a run of n histories in (at most) n_batches batches:
-// makes sure the phantom has B slabs and uploads 1/n_b; returns bs and B.
+// Batch structure of a run of n histories in (at most) n_batches batches of bs:
+// makes sure the phantom has B slabs.
 int ctx_prepare_batches(dpm_ctx *c, PhantomState *p, uint64_t n, int n_batches, uint64_t &bs, int &B);
+// Queue the fold of a run of n histories in B batches of bs.
+void ctx_fold(dpm_ctx *c, PhantomState *p, uint64_t n, uint64_t bs, int B);
 // dpm_dmax_sigma() in two halves: the kernels queued on the stream, and the wait
 // with the read-back of their n results.
 int ctx_dmax_launch(dpm_ctx *c, DmaxOut &o, const int *ids, int n);

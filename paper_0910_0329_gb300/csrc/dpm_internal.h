@@ -108,6 +108,9 @@ enum {
 // the queue kernel (counted by the warp that switches).
 constexpr int C_SWITCH = C_N;
 constexpr int kCounterSlots = C_N + 1;
+// A phantom's device counters are followed by the sum of its tally (high and low
+// halves, k_sum_tally), so that one copy brings both back.
+constexpr int kSumSlots = 2;
 
 enum { ERR_OVERFLOW = 1, ERR_STEPCAP = 2, ERR_TIMEOUT = 4 };
 

@@ -14,8 +14,11 @@ void launch_history_f64(const RunParamsT<double> &R, uint64_t batch_size, int sm
 // floats, zeroed by the caller), then their rounding into R.slabs.
 void launch_history_paper(const RunParams &R, uint64_t batch_size, bool cas, float *fslabs, size_t n_slab,
                           int sm_count, cudaStream_t st);
-void launch_fold(const unsigned long long *slabs, int nb, size_t V, const double *inv_nb, long long *S1, double *Q,
+// Fold nb batch slabs (1/inv_n histories per batch, 1/inv_n_last in the last)
+// into S1 and Q.
+void launch_fold(const unsigned long long *slabs, int nb, size_t V, double inv_n, double inv_n_last, long long *S1, double *Q,
                  int sm_count, cudaStream_t st);
+void launch_sum_tally(const long long *S1, size_t V, unsigned long long *out, int sm_count, cudaStream_t st);
 void launch_normalize(const long long *S1, const double *Q, const float *rho, size_t V, double n, double B,
                       double vox_cm3, double *dose, double *sigma, int sm_count, cudaStream_t st);
 
