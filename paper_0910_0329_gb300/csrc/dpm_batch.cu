@@ -42,7 +42,8 @@ struct Prepared {
 
 // Device work of one batch: zero the jobs' slabs, transport (one shared
 // persistent launch, then one launch per large job), fold each job.
-int batch_device_work(dpm_ctx *c, const Prepared &b, const RunParams &R, const dpm_run_opts &o, int K, int log2cs) {
+int batch_device_work(dpm_ctx *c, const Prepared &b, const RunParams &R, const dpm_run_opts &o, int K, int log2cs,
+                      int log2use) {
   for (size_t j = 0; j < b.tab.size(); ++j)
     BATCH_TRY(c, cudaMemsetAsync(b.tab[j].slabs, 0, size_t(b.nb[j]) * b.tab[j].V * sizeof(unsigned long long),
                                  c->stream));
@@ -52,11 +53,11 @@ int batch_device_work(dpm_ctx *c, const Prepared &b, const RunParams &R, const d
   std::string err;
   int rc;
   dpm_run_opts oq = o;
-  if (oq.refill_pause == 0 && log2cs < kPauseMinLog2) oq.refill_pause = -1;
-  if (!b.tab.empty() && (rc = queue_launch(c->queue.mem, K, log2cs, R, 0, oq, c->sm_count, c->stream, nullptr, err)))
+  if (oq.refill_pause == 0 && log2use < kPauseMinLog2) oq.refill_pause = -1;
+  if (!b.tab.empty() && (rc = queue_launch(c->queue.mem, K, log2cs, log2use, R, 0, oq, c->stream, nullptr, err)))
     return ctx_fail(c, rc, err);
   for (size_t j = 0; j < b.solo.size(); ++j)
-    if ((rc = queue_launch(c->queue.mem, K, log2cs, b.solo[j], b.solo_bs[j], oq, c->sm_count, c->stream, nullptr, err)))
+    if ((rc = queue_launch(c->queue.mem, K, log2cs, log2use, b.solo[j], b.solo_bs[j], oq, c->stream, nullptr, err)))
       return ctx_fail(c, rc, err);
   for (size_t j = 0; j < b.tab.size(); ++j) {
     PhantomState *p = b.ph[j];
@@ -164,9 +165,9 @@ extern "C" int dpm_run_batch(dpm_ctx *c, const dpm_job *jobs, int n_jobs, const 
   if (!b.tab.empty())
     BATCH_TRY(c, cudaMemcpyAsync(c->d_jobs, b.tab.data(), b.tab.size() * sizeof(DevJob), cudaMemcpyHostToDevice,
                                  c->stream));
-  int K = 0, log2cs = 0;
+  int K = 0, log2cs = 0, log2use = 0;
   std::string err;
-  if ((rc = queue_prepare(c->queue, o, c->sm_count, K, log2cs, err))) return ctx_fail(c, rc, err);
+  if ((rc = queue_prepare(c->queue, o, c->sm_count, c->stream, K, log2cs, log2use, err))) return ctx_fail(c, rc, err);
 
   for (RunParams &Rs : b.solo) Rs.counters = c->d_batch_counters;
   RunParams R{};
@@ -201,8 +202,9 @@ extern "C" int dpm_run_batch(dpm_ctx *c, const dpm_job *jobs, int n_jobs, const 
   c->batch_ev.push_back(ev[0]);
   c->batch_ev.push_back(ev[1]);
   if (o.use_graph) {
-    std::vector<uint64_t> sig = {uint64_t(reinterpret_cast<uintptr_t>(c->queue.mem)), uint64_t(K), uint64_t(log2cs),
-                                 uint64_t(o.refill_min), uint64_t(o.queue_limit),
+    std::vector<uint64_t> sig = {uint64_t(reinterpret_cast<uintptr_t>(c->queue.mem)), uint64_t(K), uint64_t(log2cs), uint64_t(log2use),
+                                 uint64_t(o.refill_min), uint64_t(o.refill_pause), uint64_t(o.count_events),
+                                 uint64_t(o.queue_limit),
                                  uint64_t(o.physics_flags), uint64_t(o.timeout_s * 1e6), uint64_t(b.tab.size()),
                                  uint64_t(b.total)};
     for (size_t j = 0; j < b.tab.size(); ++j) {
@@ -231,7 +233,7 @@ extern "C" int dpm_run_batch(dpm_ctx *c, const dpm_job *jobs, int n_jobs, const 
       c->batch_exec = nullptr;
       cudaGraph_t g = nullptr;
       BATCH_TRY(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-      const int wrc = batch_device_work(c, b, R, o, K, log2cs);
+      const int wrc = batch_device_work(c, b, R, o, K, log2cs, log2use);
       const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
       if (wrc) {
         if (g) cudaGraphDestroy(g);
@@ -251,7 +253,7 @@ extern "C" int dpm_run_batch(dpm_ctx *c, const dpm_job *jobs, int n_jobs, const 
     BATCH_TRY(c, cudaEventRecord(ev[1], c->stream));
   } else {
     BATCH_TRY(c, cudaEventRecord(ev[0], c->stream));
-    if ((rc = batch_device_work(c, b, R, o, K, log2cs))) return rc;
+    if ((rc = batch_device_work(c, b, R, o, K, log2cs, log2use))) return rc;
     BATCH_TRY(c, cudaEventRecord(ev[1], c->stream));
   }
   for (size_t j = 0; j < b.tab.size(); ++j) {

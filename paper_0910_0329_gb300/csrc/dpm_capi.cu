@@ -622,6 +622,7 @@ int dpm_update_phantom(dpm_ctx *c, int id, const uint8_t *mat, const float *rho)
   CUDA_TRY(c, cudaMemcpyAsync(p->d_mat, mat, p->V, cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaMemcpyAsync(p->d_rho, rho, p->V * sizeof(float), cudaMemcpyHostToDevice, c->stream));
   if ((rc = dpm_reset_tally(c, id))) return rc;
+  CUDA_TRY(c, cudaStreamSynchronize(c->stream));  // the arrays are the caller's again on return
   p->mumax_version = -1;  // new densities: the majorant must be rebuilt
   return update_mumax(c, p);
 }
@@ -636,7 +637,6 @@ int dpm_reset_tally(dpm_ctx *c, int id) {
   CUDA_TRY(c, cudaMemsetAsync(p->d_counters, 0, kCounterSlots * sizeof(unsigned long long), c->stream));
   p->n_total = 0;
   p->b_total = 0;
-  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   drop_events(p);
   return DPM_OK;
 }

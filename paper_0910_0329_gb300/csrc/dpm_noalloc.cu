@@ -88,9 +88,9 @@ extern "C" int dpm_run_noalloc(dpm_ctx *c, int phantom_id, const dpm_source *src
   if ((rc = scratch_address(&base, err))) return ctx_fail(c, rc, err);
 
   // shards that fit in the scratch, at most one per resident block
-  const int per_sm = queue_blocks_per_sm();
-  if (per_sm < 1) return ctx_fail(c, DPM_ECUDA, "occupancy query failed");
-  int K = c->sm_count * per_sm;
+  if (c->queue.per_sm < 1) c->queue.per_sm = queue_blocks_per_sm();
+  if (c->queue.per_sm < 1) return ctx_fail(c, DPM_ECUDA, "occupancy query failed");
+  int K = c->sm_count * c->queue.per_sm;
   while (K > 1 && kHeader + queue_bytes(K, kNoAllocLog2Slots) > kNoAllocBytes) --K;
   if (kHeader + queue_bytes(K, kNoAllocLog2Slots) > kNoAllocBytes)
     return ctx_fail(c, DPM_ENOMEM, "scratch too small for one queue shard");
@@ -105,7 +105,9 @@ extern "C" int dpm_run_noalloc(dpm_ctx *c, int phantom_id, const dpm_source *src
   dpm_run_opts o{};
   o.count_events = stats ? 1 : 0;
   o.refill_pause = -1;  // 512-slot shards need every refill (kPauseMinLog2)
-  if ((rc = queue_launch(hdr + kHeader, K, kNoAllocLog2Slots, R, n_histories, o, c->sm_count, c->stream, nullptr,
+  // the array is shared by every context of the process: always a fresh layout
+  if ((rc = queue_fresh(hdr + kHeader, K, kNoAllocLog2Slots, c->sm_count, c->stream, err)) ||
+      (rc = queue_launch(hdr + kHeader, K, kNoAllocLog2Slots, kNoAllocLog2Slots, R, n_histories, o, c->stream, nullptr,
                          err)))
     return ctx_fail(c, rc, err);
 

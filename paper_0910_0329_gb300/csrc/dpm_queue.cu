@@ -108,6 +108,7 @@ constexpr int kOut = 48;
 #ifndef DPM_REFILL_COOLDOWN
 #define DPM_REFILL_COOLDOWN 128
 #endif
+constexpr unsigned kSleepMaxNs = 1024;  // longest sleep of an idle warp between two looks (16 us ended launches 1 % later)
 constexpr int kSpillProbes = 8;
 
 // Where a warp looks for particles (see the refill loop of k_queue).
@@ -146,6 +147,8 @@ struct QDev {
   QType q[2];  // 0 photons, 1 electrons and positrons
   int K, log2cs;
   uint32_t mask;
+  Ctl *dirty;     // nonzero: a launch gave up a wait, the queues are not in order
+  Ctl *n_init;    // blocks of k_queue_init that are done
   Ctl *next_hist, *idle, *started;
   Ctl *backlog;   // queued particles of each type, all shards (signed; pushes add, claims subtract) [2]
   Ctl *phase;     // 0 source phase, 1 secondary phase
@@ -739,11 +742,11 @@ __device__ __forceinline__ bool idle_wait(const RunParams &R, const QDev &Q, War
       return false;
     }
     __nanosleep(sleep_ns);
-    sleep_ns = min(sleep_ns * 2, 16384u);
+    sleep_ns = min(sleep_ns * 2, kSleepMaxNs);
   }
 }
 
-__device__ void reduce_counters_q(const long long *cnt, const WarpBox *w, const RunParams &R) {
+__device__ void reduce_counters_q(const long long *cnt, const WarpBox *w, const RunParams &R, const QDev &Q) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int i = 0; i < C_N; ++i) {
@@ -752,7 +755,10 @@ __device__ void reduce_counters_q(const long long *cnt, const WarpBox *w, const 
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
     if (lane == 0 && v != 0) atomicAdd(R.counters + i, (unsigned long long)v);
   }
-  if (lane == 0 && w->err) atomicOr(R.err, w->err);
+  if (lane == 0 && w->err) {
+    atomicOr(R.err, w->err);
+    if (w->err & ERR_TIMEOUT) atomicExch(&Q.dirty->v, 1ull);
+  }
 }
 
 // Six resident blocks per SM: 24 warps with 80 registers each.  At 8 (64
@@ -893,13 +899,30 @@ __global__ void __launch_bounds__(kQBlock, DPM_QUEUE_MIN_BLOCKS)
     }
   }
   __syncwarp();
-  reduce_counters_q(sk.cnt, box, R);
+  reduce_counters_q(sk.cnt, box, R, Q);
 }
 
-__global__ void k_queue_init(uint32_t *seq0, uint32_t *seq1, size_t n, uint32_t mask) {
-  for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
-    seq0[i] = uint32_t(i) & mask;
-    seq1[i] = uint32_t(i) & mask;
+// Prepares the queues for a launch: the control words zero and, on a fresh
+// layout (`fresh`) or after a launch that gave up a wait (*dirty), the shards
+// empty.  Positions of a shard go on counting from launch to launch: a launch
+// that ends in order leaves every shard empty with its sequence words ready for
+// the next position, so nothing else has to be written.  Writing the sequence
+// words of the default queues (120 to 240 MB) before every launch, and three
+// fills, took 40 to 60 us (one 6 MV history, call and wait: 0.27 -> 0.21 ms).
+__global__ void k_queue_init(QDev Q, Ctl *ctl, int n_ctl, size_t n, bool fresh) {
+  const size_t i0 = size_t(blockIdx.x) * blockDim.x + threadIdx.x, stride = size_t(gridDim.x) * blockDim.x;
+  for (size_t i = i0; i < size_t(n_ctl); i += stride) ctl[i].v = 0;
+  if (fresh || ld_volatile(&Q.dirty->v) != 0) {
+    for (int t = 0; t < 2; ++t) {
+      for (size_t i = i0; i < size_t(Q.K); i += stride) Q.q[t].head[i].v = Q.q[t].tail[i].v = 0;
+      for (size_t i = i0; i < n; i += stride) Q.q[t].seq[i] = uint32_t(i) & Q.mask;
+    }
+  }
+  // the last block to come here, when all have read the word, clears it
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&Q.n_init->v, 1ull) == gridDim.x - 1) Q.dirty->v = Q.n_init->v = 0;
   }
 }
 
@@ -956,7 +979,9 @@ int queue_preload() {
 
 constexpr int kWordsPerSlot = 13;  // a record and its sequence word
 static_assert(sizeof(Rec) + 4 == kWordsPerSlot * 4, "record layout");
-constexpr int kCtlWords = 8 + kMaxJobs;  // next_hist idle started cur_job[2] backlog[2] phase, job_next[kMaxJobs]
+// dirty n_init | next_hist idle started cur_job[2] backlog[2] phase job_next[kMaxJobs], zeroed before every launch
+constexpr int kKeptWords = 2;
+constexpr int kCtlWords = kKeptWords + 8 + kMaxJobs;
 
 size_t queue_bytes(int K, int log2cs) {
   const size_t slots = size_t(K) << log2cs;
@@ -964,22 +989,15 @@ size_t queue_bytes(int K, int log2cs) {
   return 2 * per_type + kCtlWords * sizeof(Ctl) + 128;
 }
 
-int queue_launch(void *mem, int K, int log2cs, const RunParams &R, uint64_t batch_size, const dpm_run_opts &o,
-                 int sm_count, cudaStream_t st, cudaEvent_t start, std::string &err) {
-  if (R.jobs && (R.T.flags & DPM_SAUTER)) {
-    err = "the photoelectron angle option (DPM_SAUTER) runs in single runs only";
-    return DPM_EINVAL;
-  }
-  if (R.jobs && (R.n_jobs < 1 || R.n_jobs > kSharedJobs)) {
-    err = "a shared launch takes 1 to kSharedJobs jobs";
-    return DPM_EINVAL;
-  }
-  const size_t cs = size_t(1) << log2cs;
-  const size_t slots = size_t(K) * cs;
+// The queues of K shards of 2^log2cs slots in `mem`.
+static QDev queue_layout(void *mem, int K, int log2cs) {
+  const size_t slots = size_t(K) << log2cs;
   const size_t per_type = slots * kWordsPerSlot * sizeof(uint32_t) + 2 * size_t(K) * sizeof(Ctl);
   QDev Q{};
   char *m = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(mem) + 127) & ~uintptr_t(127));
-  Q.next_hist = reinterpret_cast<Ctl *>(m);
+  Q.dirty = reinterpret_cast<Ctl *>(m);
+  Q.n_init = Q.dirty + 1;
+  Q.next_hist = Q.dirty + kKeptWords;
   Q.idle = Q.next_hist + 1;
   Q.started = Q.next_hist + 2;
   Q.cur_job = Q.next_hist + 3;  // two words
@@ -997,7 +1015,36 @@ int queue_launch(void *mem, int K, int log2cs, const RunParams &R, uint64_t batc
   }
   Q.K = K;
   Q.log2cs = log2cs;
-  Q.mask = uint32_t(cs - 1);
+  Q.mask = uint32_t((size_t(1) << log2cs) - 1);
+  return Q;
+}
+
+int queue_fresh(void *mem, int K, int log2cs, int sm_count, cudaStream_t st, std::string &err) {
+  const QDev Q = queue_layout(mem, K, log2cs);
+  cudaError_t e = cudaMemsetAsync(Q.dirty, 0, kKeptWords * sizeof(Ctl), st);
+  if (e == cudaSuccess) {
+    k_queue_init<<<sm_count * 4, 256, 0, st>>>(Q, Q.next_hist, 0, size_t(K) << log2cs, true);
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) {
+    err = cudaGetErrorString(e);
+    return DPM_ECUDA;
+  }
+  return DPM_OK;
+}
+
+int queue_launch(void *mem, int K, int log2cs, int log2use, const RunParams &R, uint64_t batch_size,
+                 const dpm_run_opts &o, cudaStream_t st, cudaEvent_t start, std::string &err) {
+  if (R.jobs && (R.T.flags & DPM_SAUTER)) {
+    err = "the photoelectron angle option (DPM_SAUTER) runs in single runs only";
+    return DPM_EINVAL;
+  }
+  if (R.jobs && (R.n_jobs < 1 || R.n_jobs > kSharedJobs)) {
+    err = "a shared launch takes 1 to kSharedJobs jobs";
+    return DPM_EINVAL;
+  }
+  QDev Q = queue_layout(mem, K, log2cs);
+  const size_t cs = size_t(1) << log2use;
   Q.refill_min[0] = o.refill_min > 0 ? std::min(o.refill_min, 32) : DPM_REFILL_MIN_G;
   Q.refill_min[1] = o.refill_min > 0 ? std::min(o.refill_min, 32) : DPM_REFILL_MIN_E;
   Q.guard[0] = uint32_t(cs >> DPM_PHASE_GUARD_SHIFT_G);
@@ -1014,15 +1061,7 @@ int queue_launch(void *mem, int K, int log2cs, const RunParams &R, uint64_t batc
   // cost of a 20 MeV electron history on this path)
   Q.deadline_ns = Q.timeout_ns + (unsigned long long)(double(R.n) * 2000.0);
   Q.batch_size = uint32_t(batch_size);
-  // zero the control words of both types and the run counters
-  const int n_ctl = R.jobs ? 8 + R.n_jobs : 8;
-  cudaError_t e = cudaMemsetAsync(m, 0, n_ctl * sizeof(Ctl), st);
-  for (int t = 0; t < 2 && e == cudaSuccess; ++t) e = cudaMemsetAsync(Q.q[t].head, 0, 2 * size_t(K) * sizeof(Ctl), st);
-  if (e != cudaSuccess) {
-    err = cudaGetErrorString(e);
-    return DPM_ECUDA;
-  }
-  k_queue_init<<<sm_count * 4, 256, 0, st>>>(Q.q[0].seq, Q.q[1].seq, slots, Q.mask);
+  k_queue_init<<<16, 256, 0, st>>>(Q, Q.next_hist, R.jobs ? 8 + R.n_jobs : 8, size_t(K) << log2cs, false);
   if (start) cudaEventRecord(start, st);
   const bool count = o.count_events != 0;
   const bool sauter = (R.T.flags & DPM_SAUTER) != 0;
@@ -1030,7 +1069,7 @@ int queue_launch(void *mem, int K, int log2cs, const RunParams &R, uint64_t batc
   Q.pause = pause ? DPM_REFILL_COOLDOWN : 0;
   const size_t smem = R.jobs ? size_t(R.n_jobs) * sizeof(JobHot) : 0;
   queue_kernel(R.jobs != nullptr, count, sauter)<<<K, kQBlock, smem, st>>>(R, Q);
-  e = cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     err = cudaGetErrorString(e);
     return DPM_ECUDA;
@@ -1044,19 +1083,23 @@ int queue_launch(void *mem, int K, int log2cs, const RunParams &R, uint64_t batc
 // -0.3 %, so photon beams keep 2^14).
 int default_queue_log2(const RunParams &R) { return (!R.jobs && R.S.particle == 1) ? 15 : 14; }
 
-int queue_prepare(QueueState &q, const dpm_run_opts &o, int sm_count, int &K, int &log2cs, std::string &err) {
-  const int per_sm = queue_blocks_per_sm();
-  if (per_sm < 1) {
+int queue_prepare(QueueState &q, const dpm_run_opts &o, int sm_count, cudaStream_t st, int &K, int &log2cs, int &log2use,
+                  std::string &err) {
+  if (q.per_sm < 1) q.per_sm = queue_blocks_per_sm();
+  if (q.per_sm < 1) {
     err = "occupancy query failed";
     return DPM_ECUDA;
   }
-  const int bps = o.blocks_per_sm > 0 ? std::min(o.blocks_per_sm, per_sm) : per_sm;
+  const int bps = o.blocks_per_sm > 0 ? std::min(o.blocks_per_sm, q.per_sm) : q.per_sm;
   K = sm_count * bps;
-  log2cs = o.queue_log2 > 0 ? o.queue_log2 : 14;
-  if (log2cs < 7 || log2cs > 20) {
+  log2use = o.queue_log2 > 0 ? o.queue_log2 : 14;
+  if (log2use < 7 || log2use > 20) {
     err = "queue_log2 must be in [7, 20]";
     return DPM_EINVAL;
   }
+  // a layout with the same shards and room enough stays (photon and electron
+  // beams, with their 2^14 and 2^15 slots, then take turns without a new one)
+  log2cs = q.mem && q.K == K && q.log2_cap >= log2use ? q.log2_cap : log2use;
   const size_t bytes = queue_bytes(K, log2cs);
   if (q.bytes < bytes) {
     if (q.budget && q.in_use && *q.in_use - q.bytes + bytes > q.budget) {
@@ -1068,6 +1111,7 @@ int queue_prepare(QueueState &q, const dpm_run_opts &o, int sm_count, int &K, in
     if (q.in_use) *q.in_use -= q.bytes;
     q.mem = nullptr;
     q.bytes = 0;
+    q.K = 0;
     cudaError_t e = cudaMalloc(&q.mem, bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -1077,7 +1121,13 @@ int queue_prepare(QueueState &q, const dpm_run_opts &o, int sm_count, int &K, in
     q.bytes = bytes;
     if (q.in_use) *q.in_use += bytes;
   }
-  q.log2_cap = log2cs;
+  if (q.K != K || q.log2_cap != log2cs) {
+    q.K = 0;
+    const int rc = queue_fresh(q.mem, K, log2cs, sm_count, st, err);
+    if (rc) return rc;
+    q.K = K;
+    q.log2_cap = log2cs;
+  }
   return DPM_OK;
 }
 
@@ -1091,12 +1141,12 @@ int queue_run(QueueState &q, const RunParams &R, uint64_t batch_size, const dpm_
     err = "bad job count";
     return DPM_EINVAL;
   }
-  int K = 0, log2cs = 0;
+  int K = 0, log2cs = 0, log2use = 0;
   dpm_run_opts oq = o;
   if (oq.queue_log2 <= 0) oq.queue_log2 = default_queue_log2(R);
-  const int rc = queue_prepare(q, oq, sm_count, K, log2cs, err);
+  const int rc = queue_prepare(q, oq, sm_count, st, K, log2cs, log2use, err);
   if (rc) return rc;
-  return queue_launch(q.mem, K, log2cs, R, batch_size, o, sm_count, st, start, err);
+  return queue_launch(q.mem, K, log2cs, log2use, R, batch_size, o, st, start, err);
 }
 
 void queue_free(QueueState &q) {
@@ -1104,6 +1154,7 @@ void queue_free(QueueState &q) {
   if (q.in_use) *q.in_use -= q.bytes;
   q.mem = nullptr;
   q.bytes = 0;
+  q.K = 0;
 }
 
 }  // namespace dpm
