@@ -8,6 +8,13 @@
 
 namespace dpm {
 
+// What csda_energy() reads of a sink.
+struct Held {
+  float R, S;
+  __device__ float held_range() const { return R; }
+  __device__ float held_power() const { return S; }
+};
+
 __global__ void k_diag_table(DevTables T, DevPhantom P, int which, int mat, int n, const double *E, const double *aux,
                              double *out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -26,7 +33,7 @@ __global__ void k_diag_table(DevTables T, DevPhantom P, int which, int mat, int 
     case 7: r = lerp(T.pmol[size_t(mat) * T.n_e + x.i], T.pmol[size_t(mat) * T.n_e + x.i + 1], x.f); break;
     case 8: {
       const float4 a = el_at(T, mat, x);
-      r = csda_energy(T, mat, e, a.x, a.y, float(aux[i]));
+      r = csda_energy(T, mat, e, Held{a.x, a.y}, float(aux[i]));
       break;
     }
     case 9: r = lerp(P.mu_max[x.i], P.mu_max[x.i + 1], x.f); break;

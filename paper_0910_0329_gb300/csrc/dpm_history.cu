@@ -65,10 +65,17 @@ struct HistSinkT {
       pend_q = q;
     }
   }
+  __device__ __forceinline__ void leave(int) {}
   __device__ __forceinline__ void escape(Real E) { cnt[C_ESC] += fxc(E); }
-  Real held_ = Real(0);
-  __device__ __forceinline__ void hold(Real x) { held_ = x; }
-  __device__ __forceinline__ Real held() const { return held_; }
+  Real held_[3];
+  __device__ __forceinline__ void hold(Real R, Real S, Real Sigma) {
+    held_[0] = R;
+    held_[1] = S;
+    held_[2] = Sigma;
+  }
+  __device__ __forceinline__ Real held_range() const { return held_[0]; }
+  __device__ __forceinline__ Real held_power() const { return held_[1]; }
+  __device__ __forceinline__ Real held_sigma() const { return held_[2]; }
   // secondary o of particle p
   __device__ __forceinline__ void push(const PartT<Real> &p, const EmissionT<Real> &o) {
     ++cnt[C_PUSH];
@@ -242,10 +249,17 @@ struct PaperSink {
   }
   // run counters exactly as HistSink keeps them, so that the energy balance
   // of both tallies is the same
+  __device__ __forceinline__ void leave(int) {}
   __device__ __forceinline__ void escape(float E) { cnt[C_ESC] += HistSink::fxc(E); }
-  float held_ = 0.f;
-  __device__ __forceinline__ void hold(float x) { held_ = x; }
-  __device__ __forceinline__ float held() const { return held_; }
+  float held_[3];
+  __device__ __forceinline__ void hold(float R, float S, float Sigma) {
+    held_[0] = R;
+    held_[1] = S;
+    held_[2] = Sigma;
+  }
+  __device__ __forceinline__ float held_range() const { return held_[0]; }
+  __device__ __forceinline__ float held_power() const { return held_[1]; }
+  __device__ __forceinline__ float held_sigma() const { return held_[2]; }
   __device__ __forceinline__ void push(const Part &p, const Emission &o) {
     ++cnt[C_PUSH];
     if (sp < cap) {

@@ -162,7 +162,14 @@ struct QDev {
   uint32_t limit;  // pushes beyond this occupancy of a shard spill over (fault injection can lower it)
   unsigned long long timeout_ns;   // bound on any single wait
   unsigned long long deadline_ns;  // bound on the whole launch (from kernel start)
-  uint32_t batch_size;  // histories per batch (single runs)
+  // single runs: the batch of a history below 2^31 is its index divided by the
+  // batch size d, here by a multiplication: with l = ceil(log2 d) and
+  // m = ceil(2^(31+l) / d), floor(h / d) = floor(m h / 2^(31+l)) (Granlund and
+  // Montgomery, PLDI 1994); m = 0 stands for d = 1
+  uint32_t batch_mul, batch_shift;
+  __device__ __forceinline__ uint32_t batch_of(uint32_t h) const {
+    return batch_mul ? __umulhi(h, batch_mul) >> batch_shift : h;
+  }
 };
 
 __device__ __forceinline__ unsigned long long now_ns() {
@@ -228,7 +235,7 @@ struct WarpBox {
   Rec stash[kStash];  // particles of the warp's own type, for its idle lanes (last in, first out)
   Rec out[kOut];      // secondaries on their way to the queues
   long long esc[32];  // energy that left the phantom, by lane
-  float held[32];     // numbers kept for the lanes' particles (QSink::hold)
+  float held[3][32];  // numbers kept for the lanes' particles (QSink::hold)
   long long emit, miss;            // emitted and missed energy (lane 0)
   unsigned long long t_start;      // launch time of the warp
   int cool;                        // steps before the warp, with particles, looks for work again
@@ -243,8 +250,8 @@ __device__ __forceinline__ long long fxc(float e) { return __float2ll_rn(e * kCo
 // batch launch, whose particles carry their job index.  kCount: also count
 // events (steps, flights, interactions, tally atomics, pushes) for the run
 // statistics; the energy counters (emitted, escaped, missed) are always kept.
-// The event counts live in registers across the whole loop and cost about 10 %
-// of the transport rate, so runs count them only on request
+// The event counts live in registers across the whole loop and cost 3 to 8 % of
+// the transport rate, so runs count them only on request
 // (dpm_run_opts.count_events).  kSauter_: compile in the photoelectron angle
 // option (DPM_SAUTER); its code alone, unused, measured 4-6 % slower, so only
 // the single-run launches that ask for it carry it.
@@ -252,47 +259,53 @@ template <bool kMulti, bool kCount, bool kSauter_ = false>
 struct QSink {
   static constexpr bool kSauter = kSauter_;
   const RunParams &R;
+  const QDev &Q;
   const JobHot *sjobs;
   WarpBox *box;
-  uint32_t tag = 0;  // of the particle in the lane
-  int pend_v = -1;
+  uint32_t tag = 0;  // of the particle in the lane (batch launches)
+  const uint32_t *hist;  // the particle's history
   long long pend_q = 0;
   long long cnt[C_N];  // event counts only (kCount)
 
-  __device__ QSink(const RunParams &r, const JobHot *sj, WarpBox *w) : R(r), sjobs(sj), box(w) {
+  __device__ QSink(const RunParams &r, const QDev &q, const JobHot *sj, WarpBox *w, const uint32_t *h)
+      : R(r), Q(q), sjobs(sj), box(w), hist(h) {
 #pragma unroll
     for (int i = 0; i < C_N; ++i) cnt[i] = 0;
   }
   __device__ __forceinline__ static long long fx(float e) { return __float2ll_rn(e * 4294967296.0f); }
-  __device__ __forceinline__ void flush() {
-    if (pend_v >= 0 && pend_q != 0) {
+  // Run-length coalescing: a particle's deposits in one voxel are summed and
+  // added to the tally when it leaves the voxel or ends (photons, which deposit
+  // only where they interact, after the step).
+  __device__ __forceinline__ void deposit(int, float dE) { pend_q += fx(dE); }
+  __device__ __forceinline__ void leave(int v) {
+    if (pend_q != 0) {
       unsigned long long *slabs = R.slabs;
-      uint32_t V = uint32_t(R.P.nx) * uint32_t(R.P.ny) * uint32_t(R.P.nz), b = tag;
+      uint32_t V = uint32_t(R.P.nx) * uint32_t(R.P.ny) * uint32_t(R.P.nz), b;
       if (kMulti) {
-        slabs = sjobs[tag >> kTagJobShift].slabs;
-        V = sjobs[tag >> kTagJobShift].V;
+        const JobHot &J = sjobs[tag >> kTagJobShift];
+        slabs = J.slabs;
+        V = J.V;
         b = tag & ((1u << kTagJobShift) - 1);
+      } else {
+        b = Q.batch_of(*hist);
       }
-      atomicAdd(slabs + (uint64_t(b) * V + uint32_t(pend_v)), (unsigned long long)pend_q);
+      atomicAdd(slabs + (uint64_t(b) * V + uint32_t(v)), (unsigned long long)pend_q);
       if (kCount) ++cnt[C_ATOM];
-    }
-    pend_v = -1;
-    pend_q = 0;
-  }
-  __device__ __forceinline__ void deposit(int v, float dE) {
-    const long long q = fx(dE);
-    if (v == pend_v) {
-      pend_q += q;
-    } else {
-      flush();
-      pend_v = v;
-      pend_q = q;
+      pend_q = 0;
     }
   }
   __device__ __forceinline__ void escape(float E) { box->esc[threadIdx.x & 31] += fxc(E); }
   __device__ __forceinline__ void error(int e) { atomicOr(&box->err, e); }
-  __device__ __forceinline__ void hold(float x) { box->held[threadIdx.x & 31] = x; }
-  __device__ __forceinline__ float held() const { return box->held[threadIdx.x & 31]; }
+  // volatile: these are here so that no register holds them through the step
+  __device__ __forceinline__ volatile float *held_at(int k) const { return &box->held[k][threadIdx.x & 31]; }
+  __device__ __forceinline__ void hold(float R, float S, float Sigma) {
+    *held_at(0) = R;
+    *held_at(1) = S;
+    *held_at(2) = Sigma;
+  }
+  __device__ __forceinline__ float held_range() const { return *held_at(0); }
+  __device__ __forceinline__ float held_power() const { return *held_at(1); }
+  __device__ __forceinline__ float held_sigma() const { return *held_at(2); }
   __device__ __forceinline__ void count_step() {
     if (kCount) ++cnt[C_ESTEP];
   }
@@ -308,7 +321,7 @@ struct QSink {
     r.a = make_float4(p.x, p.y, p.z, o.u);
     r.b = make_float4(o.v, o.w, o.E, __uint_as_float(p.vx));
     r.c = make_uint4(o.id_lo, o.id_hi, p.hist | (o.type == POSITRON ? 0x80000000u : 0u),
-                     tag | (o.type == PHOTON ? kTagPhoton : 0u));
+                     (kMulti ? tag : 0u) | (o.type == PHOTON ? kTagPhoton : 0u));
     return r;
   }
 };
@@ -537,10 +550,10 @@ __device__ __forceinline__ bool source_exhausted(const RunParams &R, const QDev 
 // through it, the compiler would keep part of that state in local memory for
 // the whole loop and store it on every step.
 struct Parked {
-  volatile uint32_t w[17];
+  volatile uint32_t w[16];
 };
 
-__device__ __forceinline__ void park(Parked &k, const Part &p, uint32_t tag, int pend_v, long long pend_q) {
+__device__ __forceinline__ void park(Parked &k, const Part &p, uint32_t tag, long long pend_q) {
   k.w[0] = __float_as_uint(p.x);
   k.w[1] = __float_as_uint(p.y);
   k.w[2] = __float_as_uint(p.z);
@@ -555,12 +568,11 @@ __device__ __forceinline__ void park(Parked &k, const Part &p, uint32_t tag, int
   k.w[11] = p.hist;
   k.w[12] = uint32_t(p.type);
   k.w[13] = tag;
-  k.w[14] = uint32_t(pend_v);
-  k.w[15] = uint32_t(pend_q);
-  k.w[16] = uint32_t(uint64_t(pend_q) >> 32);
+  k.w[14] = uint32_t(pend_q);
+  k.w[15] = uint32_t(uint64_t(pend_q) >> 32);
 }
 
-__device__ __forceinline__ void unpark(const Parked &k, Part &p, uint32_t &tag, int &pend_v, long long &pend_q) {
+__device__ __forceinline__ void unpark(const Parked &k, Part &p, uint32_t &tag, long long &pend_q) {
   p.x = __uint_as_float(k.w[0]);
   p.y = __uint_as_float(k.w[1]);
   p.z = __uint_as_float(k.w[2]);
@@ -575,8 +587,7 @@ __device__ __forceinline__ void unpark(const Parked &k, Part &p, uint32_t &tag, 
   p.hist = k.w[11];
   p.type = int(k.w[12]);
   tag = k.w[13];
-  pend_v = int(k.w[14]);
-  const uint32_t lo = k.w[15], hi = k.w[16];
+  const uint32_t lo = k.w[14], hi = k.w[15];
   pend_q = (long long)((uint64_t(hi) << 32) | lo);
 }
 
@@ -634,8 +645,8 @@ __device__ __noinline__ int fetch_source(const RunParams &R, const QDev &Q, Warp
     w->miss += e_miss;
   }
   if (hit) {
-    const uint32_t bs = kMulti ? uint32_t(R.jobs[j].batch_size) : Q.batch_size;
-    const uint32_t tag = uint32_t(hl) / bs | (kMulti ? uint32_t(j) << kTagJobShift : 0u) | kTagPrimary;
+    uint32_t tag = kTagPrimary;
+    if (kMulti) tag |= uint32_t(hl) / uint32_t(R.jobs[j].batch_size) | uint32_t(j) << kTagJobShift;
     Rec &r = w->stash[__popc(hits & lanemask_lt())];
     r.a = make_float4(q.x, q.y, q.z, q.u);
     r.b = make_float4(q.v, q.w, q.E, __uint_as_float(q.vx));
@@ -662,7 +673,7 @@ struct Fetched {
 // grid-wide phase keeps the SMs on one of the two code paths at a time.
 template <bool kMulti>
 __device__ __forceinline__ Fetched fetch(const RunParams &R, const QDev &Q, WarpBox *w, int mode, int few, bool dry, Part &p,
-                                 uint32_t &tag, int &pend_v, long long &pend_q) {
+                                 uint32_t &tag, long long &pend_q) {
   const int S = kMulti ? current_source_type(R, Q) : (R.S.particle == 0 ? 0 : 1);
   const int O = 1 - S;
   const int ph = grid_phase(Q, S, R.counters);
@@ -684,11 +695,11 @@ __device__ __forceinline__ Fetched fetch(const RunParams &R, const QDev &Q, Warp
     if (ask == kAskSource) {
       if (source_allowed(Q, blockIdx.x % Q.K, Q.guard[S])) {
         Parked k;
-        park(k, p, tag, pend_v, pend_q);
+        park(k, p, tag, pend_q);
         const int k_src = fetch_source<kMulti>(R, Q, w, S);
         f.found = k_src >= 0;
         f.n = max(k_src, 0);
-        unpark(k, p, tag, pend_v, pend_q);
+        unpark(k, p, tag, pend_q);
         f.dry = !f.found;
         if (f.found) f.mode = S;
       }
@@ -761,10 +772,11 @@ __device__ void reduce_counters_q(const long long *cnt, const WarpBox *w, const 
   }
 }
 
-// Six resident blocks per SM: 24 warps with 80 registers each.  At 8 (64
-// registers) and 7 (72) parts of the particle's state live in local memory in
-// the hot loop (20 MeV electrons on the slabs: 683 and 476 M L2 sectors instead
-// of 309 M), 5 (96) are as fast on short launches and 7 % slower on long ones.
+// Six resident blocks per SM: 24 warps with up to 80 registers each.  Nothing
+// spills in the hot loop at 7 (72 registers) either, and it is no faster there
+// (3x10^7 6 MV histories 28.0 and 28.2 ms, 2x10^4 electrons on the slabs 0.77 and
+// 0.78 ms): more warps take more of the instruction and data caches.  8 (64
+// registers) 4 % slower, 5 as fast on short launches and 7 % slower on long ones.
 #ifndef DPM_QUEUE_MIN_BLOCKS
 #define DPM_QUEUE_MIN_BLOCKS 6
 #endif
@@ -793,8 +805,8 @@ __global__ void __launch_bounds__(kQBlock, DPM_QUEUE_MIN_BLOCKS)
     }
   }
   __syncthreads();
-  QSink<kMulti, kCount, kSauter> sk(R, sjobs, box);
   Part p{};
+  QSink<kMulti, kCount, kSauter> sk(R, Q, sjobs, box, &p.hist);
   bool alive = false;
   // warp-uniform from here on
   int n_stash = 0, n_out = 0;  // records in the stash (all of type `mode`) and in the out buffer
@@ -819,10 +831,10 @@ __global__ void __launch_bounds__(kQBlock, DPM_QUEUE_MIN_BLOCKS)
       n_out = 0;
     }
     if (look) {
-      const Fetched f = fetch<kMulti>(R, Q, box, mode, n_idle, dry, p, sk.tag, sk.pend_v, sk.pend_q);
-      n_stash = f.n;
-      mode = f.mode;
-      dry = f.dry;
+      const Fetched f = fetch<kMulti>(R, Q, box, mode, n_idle, dry, p, sk.tag, sk.pend_q);
+      n_stash = int(__reduce_max_sync(kFull, unsigned(f.n)));
+      mode = int(__reduce_max_sync(kFull, unsigned(f.mode + 1))) - 1;
+      dry = __any_sync(kFull, f.dry);
       if (lane == 0) box->cool = f.found ? 0 : Q.pause;
       __syncwarp();
     }
@@ -848,16 +860,15 @@ __global__ void __launch_bounds__(kQBlock, DPM_QUEUE_MIN_BLOCKS)
           p.hist = c.z & 0x7fffffffu;
           p.type = mode == 0 ? PHOTON : (c.z >> 31) ? POSITRON : ELECTRON;
           p.ctr = (c.w & kTagPrimary) ? 1u : 0u;
-          sk.tag = c.w & ~(kTagPhoton | kTagPrimary);
+          if (kMulti) sk.tag = c.w & ~(kTagPhoton | kTagPrimary);
           alive = true;
         }
         __syncwarp();
         n_stash = max(n_stash - n_idle, 0);
       } else if (live == 0) {
-        if (!idle_wait<kMulti>(R, Q, box)) break;
+        if (!__any_sync(kFull, idle_wait<kMulti>(R, Q, box))) break;
         p = Part{};  // nothing in the lanes: no state to keep through the wait
         sk.tag = 0;
-        sk.pend_v = -1;
         sk.pend_q = 0;
         continue;
       }
@@ -882,7 +893,7 @@ __global__ void __launch_bounds__(kQBlock, DPM_QUEUE_MIN_BLOCKS)
     // the others to the queues by way of the out buffer (which has room for 32).
     bool want = false;
     if (o.kind != EM_NONE) want = kMulti ? settle(p, o, job_step_ctx(R, sjobs, sk.tag), sk) : settle(p, o, R, sk);
-    if (was && !alive) sk.flush();
+    if (was && (!alive || mode == 0)) sk.leave(kMulti ? vox(p, job_step_ctx(R, sjobs, sk.tag).P) : vox(p, R.P));
     const unsigned all = __ballot_sync(kFull, want);
     if (all != 0) {
       if (kCount && want) ++sk.cnt[C_PUSH];
@@ -1060,7 +1071,12 @@ int queue_launch(void *mem, int K, int log2cs, int log2use, const RunParams &R, 
   // the whole launch: the wait bound plus 2 us per history (a hundred times the
   // cost of a 20 MeV electron history on this path)
   Q.deadline_ns = Q.timeout_ns + (unsigned long long)(double(R.n) * 2000.0);
-  Q.batch_size = uint32_t(batch_size);
+  if (batch_size > 1) {
+    int l = 0;
+    while ((uint64_t(1) << l) < batch_size) ++l;
+    Q.batch_mul = uint32_t(((uint64_t(1) << (31 + l)) + batch_size - 1) / batch_size);
+    Q.batch_shift = uint32_t(l - 1);
+  }
   k_queue_init<<<16, 256, 0, st>>>(Q, Q.next_hist, R.jobs ? 8 + R.n_jobs : 8, size_t(K) << log2cs, false);
   if (start) cudaEventRecord(start, st);
   const bool count = o.count_events != 0;
