@@ -84,7 +84,7 @@ extern "C" int dpm_run_batch(dpm_ctx *c, const dpm_job *jobs, int n_jobs, const 
   std::set<int> seen;
   int rc;
   // A job gets its own launch (in the same stream or graph) when its phantom
-  // and hot tally slab (13 bytes per voxel) exceed a quarter of L2 -- two
+  // and hot tally slab (16 bytes per voxel) exceed a quarter of L2 -- two
   // such jobs overlapping at a job boundary evict each other (13-15 % slower
   // on 256x256x128 phantoms) -- or when it has kSoloHistories or more: the
   // shared launch reads each particle's job record on every step and only
@@ -110,7 +110,7 @@ extern "C" int dpm_run_batch(dpm_ctx *c, const dpm_job *jobs, int n_jobs, const 
     if ((rc = ctx_prepare_batches(c, p, jobs[j].n_histories, o.n_batches, bs, B))) return rc;
     b.total += Rj.n;
     // (beyond kSharedJobs small jobs, the rest run on their own as well)
-    if (p->V * 13 > solo_bytes || jobs[j].n_histories >= kSoloHistories || int(b.tab.size()) >= kSharedJobs) {
+    if (p->V * 16 > solo_bytes || jobs[j].n_histories >= kSoloHistories || int(b.tab.size()) >= kSharedJobs) {
       Rj.n_batches = B;
       Rj.slabs = p->d_slabs;
       Rj.err = c->d_err;

@@ -94,7 +94,7 @@ void dfree(dpm_ctx *c, void *p) {
 void free_phantom(dpm_ctx *c, PhantomState *p) {
   if (!p) return;
   drop_events(p);
-  for (void *d : {(void *)p->d_mat, (void *)p->d_rho, (void *)p->d_mumax, (void *)p->d_mumax64, (void *)p->d_slabs,
+  for (void *d : {(void *)p->d_vox, (void *)p->d_mumax, (void *)p->d_mumax64, (void *)p->d_slabs,
                   (void *)p->d_fslabs,
                   (void *)p->d_S1, (void *)p->d_Q, (void *)p->d_counters, (void *)p->d_dose,
                   (void *)p->d_sigma, (void *)p->d_dmax})
@@ -225,8 +225,7 @@ static int fill_run_params(dpm_ctx *c, PhantomState *p, const dpm_source *src, u
   R.P.rdx = Real(1) / R.P.dx;
   R.P.rdy = Real(1) / R.P.dy;
   R.P.rdz = Real(1) / R.P.dz;
-  R.P.mat = p->d_mat;
-  R.P.rho = p->d_rho;
+  R.P.vox = p->d_vox;
   R.P.mu_max = mu_max;
   const double g = src->gantry_deg * 3.14159265358979323846 / 180.0;
   const double ax[3] = {std::sin(g), 0.0, std::cos(g)};
@@ -287,7 +286,7 @@ int ctx_dmax_launch(dpm_ctx *c, DmaxOut &o, const int *ids, int n) {
   // every request's result lands in one device array: one copy back
   for (int i = 0; i < n; ++i) {
     PhantomState *p = ps[i];
-    launch_dmax(p->d_S1, p->d_Q, p->d_rho, p->V, double(p->n_total), double(p->b_total), p->dx * p->dy * p->dz,
+    launch_dmax(p->d_S1, p->d_Q, p->d_vox, p->V, double(p->n_total), double(p->b_total), p->dx * p->dy * p->dz,
                 p->d_dmax, o.d + 3 * i, c->sm_count, c->stream);
   }
   CUDA_TRY(c, cudaGetLastError());
@@ -376,33 +375,44 @@ int dpm_set_stream(dpm_ctx *c, void *s) {
   return DPM_OK;
 }
 
-// Validate a phantom's host arrays; its largest material index and the
-// largest density of each material (for the photon majorant).
-static int scan_phantom(dpm_ctx *c, const uint8_t *mat, const float *rho, size_t V, int &max_mat,
-                        double (&rho_max)[DPM_MAX_MAT]) {
-  static_assert((DPM_MAX_MAT & (DPM_MAX_MAT - 1)) == 0, "material mask");
-  // one pass without branches: four partial maxima per material, so that
-  // neighbouring voxels of one material do not wait on each other's store
-  float part[4][DPM_MAX_MAT] = {};
-  unsigned bad = 0;
-  int mm = 0;
+// What is wrong with a phantom's host arrays (DPM_OK: nothing).
+static int scan_phantom(dpm_ctx *c, const uint8_t *mat, const float *rho, size_t V) {
   for (size_t v = 0; v < V; ++v) {
-    const unsigned m = mat[v];
-    const float r = rho[v];
-    bad |= unsigned(m >= DPM_MAX_MAT) | unsigned(!(r > 0.f && r <= FLT_MAX));  // also NaN and +inf
-    float &a = part[v & 3][m & (DPM_MAX_MAT - 1)];
-    a = std::max(a, r);
-    mm = std::max(mm, int(m));
+    if (mat[v] >= DPM_MAX_MAT) return fail(c, DPM_EINVAL, "material index >= 16");
+    if (!(rho[v] > 0.f) || !std::isfinite(rho[v])) return fail(c, DPM_EINVAL, "density must be positive and finite");
   }
-  if (bad) {
-    for (size_t v = 0; v < V; ++v) {
-      if (mat[v] >= DPM_MAX_MAT) return fail(c, DPM_EINVAL, "material index >= 16");
-      if (!(rho[v] > 0.f) || !std::isfinite(rho[v])) return fail(c, DPM_EINVAL, "density must be positive and finite");
-    }
+  return DPM_OK;
+}
+
+// A phantom's host arrays to the device by way of `stage` (at least 5 V bytes of
+// device memory): validated there, its largest material index and the largest
+// density of each material (for the photon majorant) noted, and packed into its
+// voxel words.  Waits, so that the arrays are the caller's again on return; with
+// an invalid array only `stage` has changed.
+static int upload_voxels(dpm_ctx *c, PhantomState *p, const uint8_t *mat, const float *rho, void *stage) {
+  float *r = static_cast<float *>(stage);
+  uint8_t *m = reinterpret_cast<uint8_t *>(r + p->V);
+  unsigned *d_scan = reinterpret_cast<unsigned *>(p->d_counters + kCounterSlots + kSumSlots);
+  unsigned scan[DPM_MAX_MAT + 1];
+  CUDA_TRY(c, cudaMemcpyAsync(r, rho, p->V * sizeof(float), cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(m, mat, p->V, cudaMemcpyHostToDevice, c->stream));
+  launch_scan_voxels(m, r, p->V, d_scan, c->sm_count, c->stream);
+  CUDA_TRY(c, cudaGetLastError());
+  CUDA_TRY(c, cudaMemcpyAsync(scan, d_scan, sizeof(scan), cudaMemcpyDeviceToHost, c->stream));
+  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  if (scan[DPM_MAX_MAT]) {
+    const int rc = scan_phantom(c, mat, rho, p->V);
+    return rc ? rc : fail(c, DPM_EINVAL, "the arrays changed during the call");
   }
-  max_mat = mm;
-  for (int m = 0; m < DPM_MAX_MAT; ++m)
-    rho_max[m] = double(std::max(std::max(part[0][m], part[1][m]), std::max(part[2][m], part[3][m])));
+  p->max_mat = 0;
+  for (int k = 0; k < DPM_MAX_MAT; ++k) {
+    float x;
+    std::memcpy(&x, scan + k, sizeof(x));
+    p->rho_max[k] = double(x);
+    if (scan[k]) p->max_mat = k;
+  }
+  launch_pack_voxels(m, r, p->V, p->d_vox, c->sm_count, c->stream);
+  CUDA_TRY(c, cudaGetLastError());
   return DPM_OK;
 }
 
@@ -419,15 +429,19 @@ int dpm_load_phantom(dpm_ctx *c, int nx, int ny, int nz, double dx, double dy, d
   p->dx = dx; p->dy = dy; p->dz = dz;
   p->V = size_t(nx) * ny * nz;
   int rc;
-  if ((rc = scan_phantom(c, mat, rho, p->V, p->max_mat, p->rho_max))) return rc;
-  if ((rc = dalloc(c, &p->d_mat, p->V)) || (rc = dalloc(c, &p->d_rho, p->V)) || (rc = dalloc(c, &p->d_S1, p->V)) ||
-      (rc = dalloc(c, &p->d_Q, p->V)) || (rc = dalloc(c, &p->d_counters, size_t(kCounterSlots + kSumSlots))) ||
+  if ((rc = dalloc(c, &p->d_vox, p->V)) || (rc = dalloc(c, &p->d_S1, p->V)) ||
+      (rc = dalloc(c, &p->d_Q, p->V)) || (rc = dalloc(c, &p->d_counters, size_t(kPhantomWords))) ||
       (rc = dalloc(c, &p->d_mumax, size_t(kMaxTableNodes)))) {
+    free_phantom(c, p.get());
+    // an invalid array is the caller's first error, with room or without
+    const int bad = scan_phantom(c, mat, rho, p->V);
+    return bad ? bad : rc;
+  }
+  // by way of the tally's memory, which is zeroed next
+  if ((rc = upload_voxels(c, p.get(), mat, rho, p->d_S1))) {
     free_phantom(c, p.get());
     return rc;
   }
-  CUDA_TRY(c, cudaMemcpyAsync(p->d_mat, mat, p->V, cudaMemcpyHostToDevice, c->stream));
-  CUDA_TRY(c, cudaMemcpyAsync(p->d_rho, rho, p->V * sizeof(float), cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaMemsetAsync(p->d_S1, 0, p->V * sizeof(long long), c->stream));
   CUDA_TRY(c, cudaMemsetAsync(p->d_Q, 0, p->V * sizeof(double), c->stream));
   CUDA_TRY(c, cudaMemsetAsync(p->d_counters, 0, kCounterSlots * sizeof(unsigned long long), c->stream));
@@ -493,7 +507,17 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
         }
     return o;
   };
-  if ((rc = upload(c, with_steps(t.ph), &ph)) || (rc = upload(c, with_steps(t.el), &el)) ||
+  // value and difference of the first component alone
+  auto first_of = [](const auto &v) {
+    std::vector<typename std::decay<decltype(v)>::type::value_type> o(v.size() / 4);
+    for (size_t k = 0; k < v.size() / 8; ++k) {
+      o[2 * k] = v[8 * k];
+      o[2 * k + 1] = v[8 * k + 4];
+    }
+    return o;
+  };
+  if ((rc = upload(c, with_steps(t.ph), &ph)) || (rc = upload(c, first_of(with_steps(t.ph)), &d.mu)) ||
+      (rc = upload(c, with_steps(t.el), &el)) ||
       (rc = upload(c, t.pmol, &d.pmol)))
     return rc;
   d.ph = reinterpret_cast<const float4 *>(ph);
@@ -532,7 +556,8 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
     d64.x_lg2 = inv * std::log(2.0);
     d64.x_lo = -std::log(t.e_lo) * inv;
     const double *ph64, *el64;
-    if ((rc = upload(c, with_steps(t.ph_64), &ph64)) || (rc = upload(c, with_steps(t.el_64), &el64)) ||
+    if ((rc = upload(c, with_steps(t.ph_64), &ph64)) || (rc = upload(c, first_of(with_steps(t.ph_64)), &d64.mu)) ||
+        (rc = upload(c, with_steps(t.el_64), &el64)) ||
         (rc = upload(c, t.pmol_64, &d64.pmol)))
       return rc;
     d64.ph = reinterpret_cast<const Dbl4 *>(ph64);
@@ -584,15 +609,14 @@ int dpm_clone_phantom(dpm_ctx *c, int src_id, int *phantom_id) {
   p->max_mat = s->max_mat;
   for (int m = 0; m < DPM_MAX_MAT; ++m) p->rho_max[m] = s->rho_max[m];
   int rc;
-  if ((rc = dalloc(c, &p->d_mat, p->V)) || (rc = dalloc(c, &p->d_rho, p->V)) || (rc = dalloc(c, &p->d_S1, p->V)) ||
-      (rc = dalloc(c, &p->d_Q, p->V)) || (rc = dalloc(c, &p->d_counters, size_t(kCounterSlots + kSumSlots))) ||
+  if ((rc = dalloc(c, &p->d_vox, p->V)) || (rc = dalloc(c, &p->d_S1, p->V)) ||
+      (rc = dalloc(c, &p->d_Q, p->V)) || (rc = dalloc(c, &p->d_counters, size_t(kPhantomWords))) ||
       (rc = dalloc(c, &p->d_mumax, size_t(kMaxTableNodes)))) {
     free_phantom(c, p.get());
     return rc;
   }
   // device-to-device, ordered on the context's stream after any pending work
-  CUDA_TRY(c, cudaMemcpyAsync(p->d_mat, s->d_mat, p->V, cudaMemcpyDeviceToDevice, c->stream));
-  CUDA_TRY(c, cudaMemcpyAsync(p->d_rho, s->d_rho, p->V * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(p->d_vox, s->d_vox, p->V * sizeof(float2), cudaMemcpyDeviceToDevice, c->stream));
   CUDA_TRY(c, cudaMemcpyAsync(p->d_mumax, s->d_mumax, kMaxTableNodes * sizeof(float), cudaMemcpyDeviceToDevice,
                               c->stream));
   p->mumax_version = s->mumax_version;
@@ -610,19 +634,16 @@ int dpm_update_phantom(dpm_ctx *c, int id, const uint8_t *mat, const float *rho)
   PhantomState *p = get_phantom(c, id);
   if (!p) return fail(c, DPM_EINVAL, "bad phantom id");
   if (!mat || !rho) return fail(c, DPM_EINVAL, "null pointer");
-  int max_mat = 0;
-  double rho_max[DPM_MAX_MAT];
-  int rc;
-  if ((rc = scan_phantom(c, mat, rho, p->V, max_mat, rho_max))) return rc;
   cudaSetDevice(c->device);
-  // earlier runs on the old contents must finish before the copies land
-  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  p->max_mat = max_mat;
-  for (int m = 0; m < DPM_MAX_MAT; ++m) p->rho_max[m] = rho_max[m];
-  CUDA_TRY(c, cudaMemcpyAsync(p->d_mat, mat, p->V, cudaMemcpyHostToDevice, c->stream));
-  CUDA_TRY(c, cudaMemcpyAsync(p->d_rho, rho, p->V * sizeof(float), cudaMemcpyHostToDevice, c->stream));
+  // The arrays are staged in the batch slabs, which hold nothing between runs
+  // (or, before the first run, in the tally, which is zero then), so that an
+  // invalid array leaves the phantom as it was.
+  int rc;
+  if ((rc = upload_voxels(c, p, mat, rho, p->d_slabs ? static_cast<void *>(p->d_slabs) : p->d_S1))) {
+    if (!p->d_slabs) CUDA_TRY(c, cudaMemsetAsync(p->d_S1, 0, p->V * sizeof(long long), c->stream));
+    return rc;
+  }
   if ((rc = dpm_reset_tally(c, id))) return rc;
-  CUDA_TRY(c, cudaStreamSynchronize(c->stream));  // the arrays are the caller's again on return
   p->mumax_version = -1;  // new densities: the majorant must be rebuilt
   return update_mumax(c, p);
 }
@@ -790,7 +811,7 @@ int dpm_read_dose(dpm_ctx *c, int id, double *dose, double *sigma, int64_t *s1_r
   if (dose || sigma) {
     int rc;
     if (!p->d_dose && ((rc = dalloc(c, &p->d_dose, p->V)) || (rc = dalloc(c, &p->d_sigma, p->V)))) return rc;
-    launch_normalize(p->d_S1, p->d_Q, p->d_rho, p->V, double(p->n_total), double(p->b_total), p->dx * p->dy * p->dz,
+    launch_normalize(p->d_S1, p->d_Q, p->d_vox, p->V, double(p->n_total), double(p->b_total), p->dx * p->dy * p->dz,
                      p->d_dose, p->d_sigma, c->sm_count, c->stream);
   }
   if (st) queue_sums(c, p);
@@ -809,7 +830,7 @@ int dpm_read_dose_device(dpm_ctx *c, int id, double *d_dose, double *d_sigma, dp
   PhantomState *p = get_phantom(c, id);
   if (!p) return fail(c, DPM_EINVAL, "bad phantom id");
   cudaSetDevice(c->device);
-  launch_normalize(p->d_S1, p->d_Q, p->d_rho, p->V, double(p->n_total), double(p->b_total), p->dx * p->dy * p->dz,
+  launch_normalize(p->d_S1, p->d_Q, p->d_vox, p->V, double(p->n_total), double(p->b_total), p->dx * p->dy * p->dz,
                    d_dose, d_sigma, c->sm_count, c->stream);
   if (st) queue_sums(c, p);
   CUDA_TRY(c, cudaGetLastError());

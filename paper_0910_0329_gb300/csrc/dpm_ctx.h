@@ -27,8 +27,7 @@ struct PhantomState {
   int nx = 0, ny = 0, nz = 0;
   double dx = 0, dy = 0, dz = 0;
   size_t V = 0;
-  uint8_t *d_mat = nullptr;
-  float *d_rho = nullptr;
+  float2 *d_vox = nullptr;  // density and material of each voxel (launch_pack_voxels)
   float *d_mumax = nullptr;  // kMaxTableNodes floats, filled for the current tables
   int mumax_version = -1;
   double *d_mumax64 = nullptr;  // the FP64 majorant (FP64 runs only), n_e doubles

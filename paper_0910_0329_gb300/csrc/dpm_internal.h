@@ -61,6 +61,7 @@ struct DevTablesT {
   // per-material tables [n_mat][n_e][2]: the node's value, then its
   // difference to the next node (zero at the last node)
   const V4 *ph;    // {mu/rho total (cm^2/g), Compton fraction, photoelectric fraction, 0}
+  const Real *mu;  // the first component alone, [n_mat][n_e][2]: what a flight reads
   const V4 *el;    // {R (g/cm^2), S (MeV cm^2/g), Sigma_hard (cm^2/g), 1/lambda1 (cm^2/g)}
   const Real *pmol;   // Moller fraction of Sigma_hard
   SampTabT<Real> kn, mol, brem, pair;
@@ -78,8 +79,7 @@ struct DevPhantomT {
   int nx, ny, nz;
   Real dx, dy, dz;
   Real rdx, rdy, rdz;  // 1/dx, 1/dy, 1/dz to the nearest
-  const uint8_t *mat;
-  const float *rho;
+  const float2 *vox;   // of each voxel: density (g/cm^3), material index (bits)
   const Real *mu_max;  // [n_e] photon majorant, 1/cm, on the tables' energy grid
 };
 
@@ -111,6 +111,9 @@ constexpr int kCounterSlots = C_N + 1;
 // A phantom's device counters are followed by the sum of its tally (high and low
 // halves, k_sum_tally), so that one copy brings both back.
 constexpr int kSumSlots = 2;
+// 64-bit words of a phantom's small device buffer: the counters, the sum, and the
+// scan of new contents (DPM_MAX_MAT + 1 32-bit words).
+constexpr int kPhantomWords = kCounterSlots + kSumSlots + (DPM_MAX_MAT + 2) / 2;
 
 enum { ERR_OVERFLOW = 1, ERR_STEPCAP = 2, ERR_TIMEOUT = 4 };
 

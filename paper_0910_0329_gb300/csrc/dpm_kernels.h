@@ -18,12 +18,15 @@ void launch_history_paper(const RunParams &R, uint64_t batch_size, bool cas, flo
 // into S1 and Q.
 void launch_fold(const unsigned long long *slabs, int nb, size_t V, double inv_n, double inv_n_last, long long *S1, double *Q,
                  int sm_count, cudaStream_t st);
+void launch_pack_voxels(const uint8_t *mat, const float *rho, size_t V, float2 *vox, int sm_count, cudaStream_t st);
+// out: DPM_MAX_MAT largest densities (bits) and an error word.
+void launch_scan_voxels(const uint8_t *mat, const float *rho, size_t V, unsigned *out, int sm_count, cudaStream_t st);
 void launch_sum_tally(const long long *S1, size_t V, unsigned long long *out, int sm_count, cudaStream_t st);
-void launch_normalize(const long long *S1, const double *Q, const float *rho, size_t V, double n, double B,
+void launch_normalize(const long long *S1, const double *Q, const float2 *vox, size_t V, double n, double B,
                       double vox_cm3, double *dose, double *sigma, int sm_count, cudaStream_t st);
 
 // D_max of the accumulated tally and its sigma: out = {dose Gy/history, sigma, voxel}.
-void launch_dmax(const long long *S1, const double *Q, const float *rho, size_t V, double n, double B, double vox_cm3,
+void launch_dmax(const long long *S1, const double *Q, const float2 *vox, size_t V, double n, double B, double vox_cm3,
                  unsigned long long *key, double *out, int sm_count, cudaStream_t st);
 
 void launch_diag_table(const DevTables &T, const DevPhantom &P, int which, int mat, int n, const double *E,

@@ -82,7 +82,7 @@ Geometry &geometry(dpm_server *s, int g) {
 // the round's batch slabs and the fixed per-phantom buffers.
 size_t slot_bytes(dpm_server *s, PhantomState *p) {
   const size_t nb = size_t(s->o.n_batches);
-  return p->V * (1 + 4 + 8 + 8 + 8 * nb) + kMaxTableNodes * 4 + 16384;
+  return p->V * (8 + 8 + 8 + 8 * nb) + kMaxTableNodes * 4 + 16384;
 }
 
 Geometry &sized_geometry(dpm_server *s, int g) {
