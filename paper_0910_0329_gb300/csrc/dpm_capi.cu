@@ -490,34 +490,29 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
   }
   int rc;
   const float *ph, *el;
-  // device layout of the float4 tables: each node's value followed by the
-  // float difference to the next node (see el_at in dpm_device.cuh)
-  auto with_steps = [&](const auto &h) {
-    using T = typename std::decay<decltype(h)>::type::value_type;
-    std::vector<T> o(2 * h.size(), T(0));
-    for (int m = 0; m < t.n_mat; ++m)
-      for (int i = 0; i < t.n_e; ++i)
-        for (int k = 0; k < 4; ++k) {
-          const size_t at = (size_t(m) * t.n_e + i) * 4 + k;
-          o[2 * at - k] = h[at];
-          if (i + 1 < t.n_e) {
-            volatile T diff = h[at + 4] - h[at];  // one subtraction in the table's type, as on the device
-            o[2 * at - k + 4] = diff;
-          }
-        }
-    return o;
+  // An interpolation reads its node and the next.  One more node, a copy of the
+  // last, stands behind the last material: in FP32 the position's upper clamp
+  // reaches the last node itself from 32770 nodes up.
+  auto padded = [](auto h) {
+    for (int k = 0; k < 4; ++k) h.push_back(h[h.size() - 4]);
+    return h;
   };
-  // value and difference of the first component alone
-  auto first_of = [](const auto &v) {
-    std::vector<typename std::decay<decltype(v)>::type::value_type> o(v.size() / 4);
-    for (size_t k = 0; k < v.size() / 8; ++k) {
-      o[2 * k] = v[8 * k];
-      o[2 * k + 1] = v[8 * k + 4];
+  // the photon table's first component with its difference to the next node
+  // (zero at the last), one aligned pair for a flight
+  auto pairs_of = [&](const auto &h) {
+    using T = typename std::decay<decltype(h)>::type::value_type;
+    std::vector<T> o(h.size() / 2, T(0));
+    for (size_t k = 0; k < o.size() / 2; ++k) {
+      o[2 * k] = h[4 * k];
+      if ((k + 1) % t.n_e) {
+        volatile T diff = h[4 * k + 4] - h[4 * k];  // one subtraction in the table's type, as on the device
+        o[2 * k + 1] = diff;
+      }
     }
     return o;
   };
-  if ((rc = upload(c, with_steps(t.ph), &ph)) || (rc = upload(c, first_of(with_steps(t.ph)), &d.mu)) ||
-      (rc = upload(c, with_steps(t.el), &el)) ||
+  if ((rc = upload(c, padded(t.ph), &ph)) || (rc = upload(c, pairs_of(t.ph), &d.mu)) ||
+      (rc = upload(c, padded(t.el), &el)) ||
       (rc = upload(c, t.pmol, &d.pmol)))
     return rc;
   d.ph = reinterpret_cast<const float4 *>(ph);
@@ -556,8 +551,8 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
     d64.x_lg2 = inv * std::log(2.0);
     d64.x_lo = -std::log(t.e_lo) * inv;
     const double *ph64, *el64;
-    if ((rc = upload(c, with_steps(t.ph_64), &ph64)) || (rc = upload(c, first_of(with_steps(t.ph_64)), &d64.mu)) ||
-        (rc = upload(c, with_steps(t.el_64), &el64)) ||
+    if ((rc = upload(c, padded(t.ph_64), &ph64)) || (rc = upload(c, pairs_of(t.ph_64), &d64.mu)) ||
+        (rc = upload(c, padded(t.el_64), &el64)) ||
         (rc = upload(c, t.pmol_64, &d64.pmol)))
       return rc;
     d64.ph = reinterpret_cast<const Dbl4 *>(ph64);

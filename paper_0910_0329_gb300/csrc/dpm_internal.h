@@ -58,10 +58,9 @@ struct DevTablesT {
   int n_mat, n_e;
   Real lnE_lo, inv_dlnE;
   Real x_lg2, x_lo;  // grid position = log2(E) * x_lg2 + x_lo
-  // per-material tables [n_mat][n_e][2]: the node's value, then its
-  // difference to the next node (zero at the last node)
+  // per-material tables [n_mat][n_e], and one node more
   const V4 *ph;    // {mu/rho total (cm^2/g), Compton fraction, photoelectric fraction, 0}
-  const Real *mu;  // the first component alone, [n_mat][n_e][2]: what a flight reads
+  const Real *mu;  // the first component alone, [n_mat][n_e][2]: value, difference to the next node (0 at the last)
   const V4 *el;    // {R (g/cm^2), S (MeV cm^2/g), Sigma_hard (cm^2/g), 1/lambda1 (cm^2/g)}
   const Real *pmol;   // Moller fraction of Sigma_hard
   SampTabT<Real> kn, mol, brem, pair;
