@@ -222,6 +222,9 @@ static int fill_run_params(dpm_ctx *c, PhantomState *p, const dpm_source *src, u
   R.P.dx = Real(p->dx);
   R.P.dy = Real(p->dy);
   R.P.dz = Real(p->dz);
+  R.P.X = Real(R.P.nx) * R.P.dx;
+  R.P.Y = Real(R.P.ny) * R.P.dy;
+  R.P.Z = Real(R.P.nz) * R.P.dz;
   R.P.rdx = Real(1) / R.P.dx;
   R.P.rdy = Real(1) / R.P.dy;
   R.P.rdz = Real(1) / R.P.dz;
@@ -518,8 +521,9 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
   d.ph = reinterpret_cast<const float4 *>(ph);
   d.el = reinterpret_cast<const float4 *>(el);
   auto samp = [&](const std::vector<float> &v, int ne, double lo, double hi, SampTab &s) {
-    s.ne = ne;
+    s.x_top = float(ne - 1) - 1e-3f;
     s.nu = t.nu;
+    s.y_top = float(t.nu - 1);
     s.lnE0 = float(std::log(lo));
     s.inv_dlnE = float((ne - 1) / (std::log(hi) - std::log(lo)));
     return upload(c, v, &s.y);
@@ -529,9 +533,11 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
       (rc = samp(t.pair, t.pair_ne, t.pair_lo, t.pair_hi, d.pair)) || (rc = upload(c, t.msc, &d.msc_lnA)) ||
       (rc = samp(t.sauter, t.sauter_ne, t.sauter_lo, t.sauter_hi, d.sauter)))
     return rc;
-  d.msc_n = t.msc_n;
   d.msc_x0 = float(t.msc_x0);
   d.msc_inv_dx = float((t.msc_n - 1) / (t.msc_x1 - t.msc_x0));
+  d.msc_top = float(t.msc_n - 1);
+  d.msc_x1 = d.msc_x0 + d.msc_top / d.msc_inv_dx;
+  d.x_top = float(t.n_e - 1) - 1e-3f;
   d.eabs_e = float(p->eabs_e);
   d.eabs_g = float(p->eabs_g);
   d.wcc = float(p->wcc);
@@ -558,8 +564,9 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
     d64.ph = reinterpret_cast<const Dbl4 *>(ph64);
     d64.el = reinterpret_cast<const Dbl4 *>(el64);
     auto samp64 = [&](const std::vector<double> &v, int ne, double lo, double hi, SampTabT<double> &s) {
-      s.ne = ne;
+      s.x_top = double(ne - 1) - double(1e-3f);
       s.nu = t.nu;
+      s.y_top = double(t.nu - 1);
       s.lnE0 = std::log(lo);
       s.inv_dlnE = (ne - 1) / (std::log(hi) - std::log(lo));
       return upload(c, v, &s.y);
@@ -571,9 +578,11 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
         (rc = upload(c, t.msc_64, &d64.msc_lnA)) ||
         (rc = samp64(t.sauter_64, t.sauter_ne, t.sauter_lo, t.sauter_hi, d64.sauter)))
       return rc;
-    d64.msc_n = t.msc_n;
     d64.msc_x0 = t.msc_x0;
     d64.msc_inv_dx = (t.msc_n - 1) / (t.msc_x1 - t.msc_x0);
+    d64.msc_top = double(t.msc_n - 1);
+    d64.msc_x1 = d64.msc_x0 + d64.msc_top / d64.msc_inv_dx;
+    d64.x_top = double(t.n_e - 1) - double(1e-3f);
     d64.eabs_e = p->eabs_e;
     d64.eabs_g = p->eabs_g;
     d64.wcc = p->wcc;

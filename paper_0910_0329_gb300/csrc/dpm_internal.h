@@ -47,7 +47,8 @@ struct Vec4<double> {
 template <class Real>
 struct SampTabT {
   const Real *y;  // [ne][nu]
-  int ne, nu;
+  int nu;
+  Real x_top, y_top;  // largest energy position (ne - 1 - 1e-3), nu - 1
   Real lnE0, inv_dlnE;
 };
 
@@ -55,9 +56,13 @@ struct SampTabT {
 template <class Real>
 struct DevTablesT {
   using V4 = typename Vec4<Real>::type;
+  // What a step needs of the sizes stands here as Real, in every struct of this
+  // view: the kernels have no registers to keep it in, and converted (or, for
+  // msc_x1, divided) it again at each use (1.5 % of the 20 MeV runs).
   int n_mat, n_e;
   Real lnE_lo, inv_dlnE;
   Real x_lg2, x_lo;  // grid position = log2(E) * x_lg2 + x_lo
+  Real x_top;        // largest position, n_e - 1 - 1e-3
   // per-material tables [n_mat][n_e], and one node more
   const V4 *ph;    // {mu/rho total (cm^2/g), Compton fraction, photoelectric fraction, 0}
   const Real *mu;  // the first component alone, [n_mat][n_e][2]: value, difference to the next node (0 at the last)
@@ -65,8 +70,8 @@ struct DevTablesT {
   const Real *pmol;   // Moller fraction of Sigma_hard
   SampTabT<Real> kn, mol, brem, pair;
   const Real *msc_lnA;  // ln A on a uniform grid of logit(q)
-  int msc_n;
   Real msc_x0, msc_inv_dx;
+  Real msc_top, msc_x1;  // last node, msc_x0 + msc_top / msc_inv_dx
   Real eabs_e, eabs_g, wcc, wcr, f_e;
   int flags;  // DPM_NO_HARD / DPM_NO_MSC
   Real x_fe, x_eabs;  // grid-index shift of an energy step (1 - f_e), grid index of eabs_e
@@ -78,6 +83,7 @@ struct DevPhantomT {
   int nx, ny, nz;
   Real dx, dy, dz;
   Real rdx, rdy, rdz;  // 1/dx, 1/dy, 1/dz to the nearest
+  Real X, Y, Z;        // the phantom's size: nx dx and so on, in Real
   const float2 *vox;   // of each voxel: density (g/cm^3), material index (bits)
   const Real *mu_max;  // [n_e] photon majorant, 1/cm, on the tables' energy grid
 };
