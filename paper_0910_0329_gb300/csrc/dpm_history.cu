@@ -73,6 +73,7 @@ struct HistSinkT {
     held_[1] = S;
     held_[2] = Sigma;
   }
+  static __device__ __forceinline__ bool hard_waits() { return false; }
   __device__ __forceinline__ Real held_range() const { return held_[0]; }
   __device__ __forceinline__ Real held_power() const { return held_[1]; }
   __device__ __forceinline__ Real held_sigma() const { return held_[2]; }
@@ -257,6 +258,7 @@ struct PaperSink {
     held_[1] = S;
     held_[2] = Sigma;
   }
+  static __device__ __forceinline__ bool hard_waits() { return false; }
   __device__ __forceinline__ float held_range() const { return held_[0]; }
   __device__ __forceinline__ float held_power() const { return held_[1]; }
   __device__ __forceinline__ float held_sigma() const { return held_[2]; }

@@ -96,6 +96,16 @@ constexpr int kStealProbes = DPM_STEAL_PROBES;
 #ifndef DPM_FETCH_MIN
 #define DPM_FETCH_MIN 8
 #endif
+// Calls of electron_step between two that make hard events: an event is some 300
+// instructions with its secondary, and one or two lanes of a warp have one in
+// half of all calls.  Waiting in its lane for the next such call it meets
+// others: 5x10^6 20 MeV electrons on the 128^3 blobs 30.8 (every call), 29.9
+// (every 2nd), 28.9 (4th), 28.9 (8th) ms; 2x10^4 on the slab 0.70, 0.68, 0.67,
+// 0.68 ms.
+#ifndef DPM_HARD_EVERY
+#define DPM_HARD_EVERY 4
+#endif
+constexpr unsigned kHardEvery = DPM_HARD_EVERY;
 // Records of a warp's stash and of its out buffer, which always has room for a
 // step's 32.  Larger ones (48, 64) measured the same.
 constexpr int kStash = 32;
@@ -265,6 +275,8 @@ struct QSink {
   uint32_t tag = 0;  // of the particle in the lane (batch launches)
   const uint32_t *hist;  // the particle's history
   long long pend_q = 0;
+  unsigned calls = 0;  // of the warp (uniform)
+  __device__ __forceinline__ bool hard_waits() const { return calls % kHardEvery != 0; }
   long long cnt[C_N];  // event counts only (kCount)
 
   __device__ QSink(const RunParams &r, const QDev &q, const JobHot *sj, WarpBox *w, const uint32_t *h)
@@ -764,13 +776,13 @@ __device__ void reduce_counters_q(const long long *cnt, const WarpBox *w, const 
   }
 }
 
-// Six resident blocks per SM: 24 warps with up to 80 registers each.  Nothing
-// spills in the hot loop at 7 (72 registers) either, and it is no faster there
-// (3x10^7 6 MV histories 28.0 and 28.2 ms, 2x10^4 electrons on the slabs 0.77 and
-// 0.78 ms): more warps take more of the instruction and data caches.  8 (64
-// registers) 4 % slower, 5 as fast on short launches and 7 % slower on long ones.
+// Seven resident blocks per SM: 28 warps with up to 72 registers each, and
+// nothing spilled in the hot loop.  6, 7 and 8 blocks (80, 72 and 64 registers):
+// 10^7 6 MV histories 9.68, 8.83 and 9.98 ms, 5x10^6 20 MeV electrons on the
+// 128^3 blobs 28.9, 26.4 and 29.8 ms, 2x10^4 on the slab 0.57, 0.58 and 0.70 ms.
+// (6 blocks that are held to 72 registers: 9.29, 28.1 and 0.56 ms.)
 #ifndef DPM_QUEUE_MIN_BLOCKS
-#define DPM_QUEUE_MIN_BLOCKS 6
+#define DPM_QUEUE_MIN_BLOCKS 7
 #endif
 template <bool kMulti, bool kCount, bool kSauter = false>
 __global__ void __launch_bounds__(kQBlock, DPM_QUEUE_MIN_BLOCKS)
@@ -866,6 +878,7 @@ __global__ void __launch_bounds__(kQBlock, DPM_QUEUE_MIN_BLOCKS)
       }
     }
     const bool was = alive;
+    ++sk.calls;
     Emission o;
     if (alive) {
       if (p.type & CHAIN)
@@ -949,7 +962,7 @@ QKernel queue_kernel(bool multi, bool count, bool sauter) {
 }
 
 int queue_blocks_per_sm() {
-  // Shared memory for the resident blocks (17 KB of stashes and buffers each,
+  // Shared memory for the resident blocks (18 KB of stashes and buffers each,
   // in a batch launch also the step records of up to kSharedJobs jobs, and 1 KB
   // reserved), the rest to L1, where the tables are cached.
   int best = 1 << 30;
@@ -958,7 +971,7 @@ int queue_blocks_per_sm() {
     int per_sm = 0;
     const bool multi = e.multi;
     const size_t smem = multi ? kSharedJobs * sizeof(JobHot) : 0;
-    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, multi ? 64 : 50);
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, multi ? 80 : 58);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kQBlock, smem) != cudaSuccess) {
       cudaGetLastError();
       return 0;
