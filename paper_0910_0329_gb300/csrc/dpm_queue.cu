@@ -111,10 +111,16 @@ constexpr int kStealProbes = DPM_STEAL_PROBES;
 #define DPM_HARD_EVERY 4
 #endif
 constexpr unsigned kHardEvery = DPM_HARD_EVERY;
-// Records of a warp's stash and of its out buffer, which always has room for a
-// step's 32.  Larger ones (48, 64) measured the same.
+// Records of a warp's stash and of its out buffer, and how many in the buffer
+// are sent to the queues by a warp of photons and one of electrons: the buffer
+// has room for a step's 32 always.  Sending is a chain of four L2 round trips,
+// and the 17 electrons that a call of a full photon warp leaves on the slab
+// phantom went to the queues in nearly every call while 16 were kept; now 32 go
+// at a time (10^7 6 MV histories 8.44 -> 8.29 ms; 24 kept: 8.38).  An electron
+// warp leaves a photon or two per call, which other warps may be waiting for.
 constexpr int kStash = 32;
-constexpr int kOut = 48;
+constexpr int kOut = 64;
+constexpr int kKeepG = 32, kKeepE = 16;
 // Fetch pause: a warp with particles waits this many steps, after it found no
 // work for its stash, before it looks again.  A look costs several dependent L2
 // round trips, and in the phase of the other type, or at the end of a launch,
@@ -367,13 +373,13 @@ __device__ __forceinline__ int reserve(const QDev &Q, int t, int n, unsigned lon
   return -1;
 }
 
-// Queue the n records of the warp's out buffer: one atomic per 32 records on
+// Queue records [from, n) of the warp's out buffer: one atomic per 32 records on
 // the shard's tail and the backlog of each type.
-__device__ __forceinline__ void flush_out(const QDev &Q, WarpBox *w, int n) {
+__device__ __forceinline__ void flush_out(const QDev &Q, WarpBox *w, int from, int n) {
   const int lane = threadIdx.x & 31;
   __syncwarp();
 #pragma unroll 1
-  for (int i = lane; i - lane < n; i += 32) {
+  for (int i = from + lane; i - lane < n; i += 32) {
     const bool have = i < n;
     const int t = have && (w->out[i].c.w & kTagPhoton) ? 0 : 1;
     const unsigned m0 = __ballot_sync(kFull, have && t == 0), m1 = __ballot_sync(kFull, have && t == 1);
@@ -825,7 +831,7 @@ __global__ void __launch_bounds__(kQBlock, DPM_QUEUE_MIN_BLOCKS)
     const unsigned live = __ballot_sync(kFull, alive);
     const int n_idle = 32 - __popc(live);
     // near the end of a launch every particle is for whoever is idle
-    const bool send = n_out > kOut - 32 || (n_out != 0 && (dry || live == 0));
+    const bool send = n_out > (mode == 0 ? kKeepG : kKeepE) || (n_out != 0 && (dry || live == 0));
     bool look = live == 0 && n_stash == 0;
     if (live == 0 && n_stash == 0) {
       mode = -1;
@@ -836,8 +842,9 @@ __global__ void __launch_bounds__(kQBlock, DPM_QUEUE_MIN_BLOCKS)
       look = c == 0;
     }
     if (send) {
-      flush_out(Q, box, n_out);
-      n_out = 0;
+      const int from = dry || live == 0 ? 0 : max(n_out - 32, 0);  // the newest 32, or all
+      flush_out(Q, box, from, n_out);
+      n_out = from;
     }
     if (look) {
       const Fetched f = fetch<kMulti>(R, Q, box, mode, n_idle, dry, p, sk.tag, sk.pend_q);
@@ -967,16 +974,17 @@ QKernel queue_kernel(bool multi, bool count, bool sauter) {
 }
 
 int queue_blocks_per_sm() {
-  // Shared memory for the resident blocks (18 KB of stashes and buffers each,
+  // Shared memory for the resident blocks (21 KB of stashes and buffers each,
   // in a batch launch also the step records of up to kSharedJobs jobs, and 1 KB
-  // reserved), the rest to L1, where the tables are cached.
+  // reserved), the rest to L1, where the tables are cached: at 84 % for batch
+  // launches, which takes the next larger split, serving took 5 % longer.
   int best = 1 << 30;
   for (const QKernelEntry &e : kQueueKernels) {
     const QKernel k = e.k;
     int per_sm = 0;
     const bool multi = e.multi;
     const size_t smem = multi ? kSharedJobs * sizeof(JobHot) : 0;
-    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, multi ? 80 : 58);
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, multi ? 80 : 70);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kQBlock, smem) != cudaSuccess) {
       cudaGetLastError();
       return 0;
