@@ -24,24 +24,25 @@
 // is bounded by a time limit read from %globaltimer; on expiry the kernel
 // records an error and returns.
 //
-// What bounds the kernel: instruction issue, instruction fetch and the latency
-// of table lookups, not memory bandwidth.  Three things follow.
+// What bounds the kernel: instruction issue (73 to 78 % of the slots on long
+// launches, at 21 of 32 lanes), then instruction fetch and the latency of table
+// lookups, not memory bandwidth.  Four things follow.
 // - Code size.  The kernel took 276 KB when every secondary was queued where it
 //   is made, every refill was spelled out and the photon interaction stood
 //   after each of two flights; "no instruction" was the leading stall (4.7 of
 //   17 cycles per issue on 6 MV, 5.0 on 20 MeV electrons).  With one copy of
-//   each it takes 83 KB (2.1 and 2.0 cycles).
+//   each it takes 81 KB (1.2 and 1.7 cycles).
 // - Full warps.  Lanes that wait for a refill waste issue slots, and a refill
 //   from the device-wide queues costs several L2 round trips.  Taking from the
-//   stash costs some 60 instructions, so it happens at 2 idle lanes: 28.5
-//   (photons) and 28.7 (electrons) of 32 lanes carry particles on 3x10^7 6 MV
-//   histories, against 19.1 and 25.5 with refills from the queues at 24 and 12
-//   idle lanes.
+//   stash costs some 60 instructions, so it happens at 2 idle lanes.  What few
+//   lanes of a warp do at a time waits for company: see kHardEvery.
 // - Few instructions per step: see Num<float> and electron_step in
 //   dpm_device.cuh.
-// Transport times, before and with all three: 10^7 6 MV histories 14.6 and
-// 10.1 ms, 5x10^6 20 MeV electrons on the 128^3 blobs 52.4 and 33.2 ms, 2x10^4
-// on the slabs 1.58 and 0.79 ms, 2000 photons of 15 MeV 0.63 and 0.47 ms.
+// - Nothing at the ends of a launch that grows with the grid: see any_work and
+//   queue_fresh.
+// Transport times, before and with all four: 10^7 6 MV histories 14.6 and
+// 8.3 ms, 5x10^6 20 MeV electrons on the 128^3 blobs 52.4 and 25.8 ms, 2x10^4
+// on the slabs 1.58 and 0.59 ms, 2000 photons of 15 MeV 0.63 and 0.34 ms.
 #include <cuda_runtime.h>
 
 #include "dpm_device.cuh"
