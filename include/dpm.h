@@ -145,8 +145,10 @@ typedef struct {
                           step (-1); 0 = automatic: the pause, but none with queue
                           shards below 2^13 slots (queue_log2 < 13, or
                           dpm_run_noalloc's), which need every refill to keep from
-                          overflowing.  Scheduling only: the tally is the same either
-                          way, unless a queue overflows. */
+                          overflowing.  With shards below 2^9 slots a warp looks only
+                          when it has no particles, whatever this says.  Scheduling
+                          only: the tally is the same either way, unless a queue
+                          overflows. */
 } dpm_run_opts;
 enum { DPM_NO_HARD = 1, DPM_NO_MSC = 2, DPM_SAUTER = 4 };
 

@@ -102,6 +102,14 @@ constexpr int kStealProbes = DPM_STEAL_PROBES;
 #ifndef DPM_FETCH_MIN
 #define DPM_FETCH_MIN 8
 #endif
+// On shards below 2^kFullFetchLog2 slots a warp fetches only when it is empty (its
+// pause after a fetch outlasts its particles), and a photon beam's secondary phase
+// starts at half the backlog: with photons in the stash as well as in the lanes,
+// what they still leave after their phase has ended is more than such a shard holds
+// (six photon beams of 10^5 to 5x10^6 histories on 256-slot shards: 108 of 240 runs
+// overflowed, now none; without stashes 1 of 240).  Runs on larger shards take the
+// same time as before (within 0.2 %).
+constexpr int kFullFetchLog2 = 9;
 // Calls of electron_step between two that make hard events: an event is some 300
 // instructions with its secondary, and one or two lanes of a warp have one in
 // half of all calls.  Waiting in its lane for the next such call it meets
@@ -178,7 +186,7 @@ struct QDev {
                   // start (word 0; word 1 unused)
   Ctl *job_next;  // batch launches: next history of each job [kMaxJobs]
   int refill_min[2];  // idle lanes before a warp takes from its stash, by its particle type (photon, electron)
-  int pause;          // steps a warp with particles waits after a fetch that found none
+  int pause[2];       // steps a warp with particles waits after a fetch that found none, some
   uint32_t guard[2];               // per-shard bound for sources, by beam type
   long long phase_high[2], phase_low[2];  // global backlog thresholds, by beam type
   uint32_t limit;  // pushes beyond this occupancy of a shard spill over (fault injection can lower it)
@@ -676,8 +684,8 @@ struct Fetched {
 };
 
 // Fill the empty stash of a warp of type `mode` (-1: no particles in its lanes)
-// with up to 32 particles, or `few` once the source is dry: near the end of a
-// launch the queued particles are spread over the warps.
+// with up to 32 particles, or `few` (its idle lanes) once the source is dry: near
+// the end of a launch the queued particles are spread over the warps.
 //
 // Source phase: warps start histories and track particles of the beam's type
 // while the secondaries of the other type pile up in the queues; secondary
@@ -852,7 +860,7 @@ __global__ void __launch_bounds__(kQBlock, DPM_QUEUE_MIN_BLOCKS)
       n_stash = int(__reduce_max_sync(kFull, unsigned(f.n)));
       mode = int(__reduce_max_sync(kFull, unsigned(f.mode + 1))) - 1;
       dry = __any_sync(kFull, f.dry);
-      if (lane == 0) box->cool = f.found ? 0 : Q.pause;
+      if (lane == 0) box->cool = Q.pause[f.found ? 1 : 0];
       __syncwarp();
     }
     if (n_idle >= Q.refill_min[mode > 0 ? 1 : 0] || live == 0) {
@@ -1077,9 +1085,10 @@ int queue_launch(void *mem, int K, int log2cs, int log2use, const RunParams &R, 
   const size_t cs = size_t(1) << log2use;
   Q.refill_min[0] = o.refill_min > 0 ? std::min(o.refill_min, 32) : DPM_REFILL_MIN_G;
   Q.refill_min[1] = o.refill_min > 0 ? std::min(o.refill_min, 32) : DPM_REFILL_MIN_E;
-  Q.guard[0] = uint32_t(cs >> DPM_PHASE_GUARD_SHIFT_G);
+  const bool small = log2use < kFullFetchLog2;
+  Q.guard[0] = uint32_t(cs >> (small ? 2 : DPM_PHASE_GUARD_SHIFT_G));
   Q.guard[1] = uint32_t(cs >> DPM_PHASE_GUARD_SHIFT_E);
-  Q.phase_high[0] = (long long)K * (long long)(cs >> DPM_PHASE_HIGH_SHIFT_G);
+  Q.phase_high[0] = (long long)K * (long long)(cs >> (small ? 3 : DPM_PHASE_HIGH_SHIFT_G));
   // at least one particle per shard: a phase that ended below 0 would never end
   Q.phase_low[0] = (long long)K * (long long)std::max(cs >> DPM_PHASE_LOW_SHIFT_G, decltype(cs)(1));
   Q.phase_high[1] = (long long)K * (long long)(cs >> DPM_PHASE_HIGH_SHIFT_E);
@@ -1102,7 +1111,8 @@ int queue_launch(void *mem, int K, int log2cs, int log2use, const RunParams &R, 
   const bool count = o.count_events != 0;
   const bool sauter = (R.T.flags & DPM_SAUTER) != 0;
   const bool pause = o.refill_pause >= 0;  // callers on queues below 2^kPauseMinLog2 slots pass -1 for 0
-  Q.pause = pause ? DPM_REFILL_COOLDOWN : 0;
+  Q.pause[0] = small ? 1 << 30 : pause ? DPM_REFILL_COOLDOWN : 0;
+  Q.pause[1] = small ? 1 << 30 : 0;
   const size_t smem = R.jobs ? size_t(R.n_jobs) * sizeof(JobHot) : 0;
   queue_kernel(R.jobs != nullptr, count, sauter)<<<K, kQBlock, smem, st>>>(R, Q);
   const cudaError_t e = cudaGetLastError();
