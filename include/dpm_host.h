@@ -24,7 +24,8 @@ void dpm_host_tables_free(void *handle);
 /* Copy table `name` ("ph", "el", "pmol", "kn", "mol", "brem", "pair", "msc")
    into out (at most n floats; out may be NULL to query the length).  meta
    (6 doubles, may be NULL) receives [e_lo, e_hi, rows or nodes, row or
-   argument range lo, hi, columns].  Returns the table length or -1. */
+   argument range lo, hi, columns]; for "ph", "el" and "pmol" the range is that
+   of the positions, in nodes, at which the kernels read them.  Returns the table length or -1. */
 int dpm_host_tables_get(void *handle, const char *name, float *out, int n, double *meta);
 
 #ifdef __cplusplus

@@ -493,13 +493,6 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
   }
   int rc;
   const float *ph, *el;
-  // An interpolation reads its node and the next.  One more node, a copy of the
-  // last, stands behind the last material: in FP32 the position's upper clamp
-  // reaches the last node itself from 32770 nodes up.
-  auto padded = [](auto h) {
-    for (int k = 0; k < 4; ++k) h.push_back(h[h.size() - 4]);
-    return h;
-  };
   // the photon table's first component with its difference to the next node
   // (zero at the last), one aligned pair for a flight
   auto pairs_of = [&](const auto &h) {
@@ -514,14 +507,14 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
     }
     return o;
   };
-  if ((rc = upload(c, padded(t.ph), &ph)) || (rc = upload(c, pairs_of(t.ph), &d.mu)) ||
-      (rc = upload(c, padded(t.el), &el)) ||
+  if ((rc = upload(c, t.ph, &ph)) || (rc = upload(c, pairs_of(t.ph), &d.mu)) ||
+      (rc = upload(c, t.el, &el)) ||
       (rc = upload(c, t.pmol, &d.pmol)))
     return rc;
   d.ph = reinterpret_cast<const float4 *>(ph);
   d.el = reinterpret_cast<const float4 *>(el);
   auto samp = [&](const std::vector<float> &v, int ne, double lo, double hi, SampTab &s) {
-    s.x_top = float(ne - 1) - 1e-3f;
+    s.x_top = grid_top<float>(ne);
     s.nu = t.nu;
     s.y_top = float(t.nu - 1);
     s.lnE0 = float(std::log(lo));
@@ -537,7 +530,7 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
   d.msc_inv_dx = float((t.msc_n - 1) / (t.msc_x1 - t.msc_x0));
   d.msc_top = float(t.msc_n - 1);
   d.msc_x1 = d.msc_x0 + d.msc_top / d.msc_inv_dx;
-  d.x_top = float(t.n_e - 1) - 1e-3f;
+  d.x_top = grid_top<float>(t.n_e);
   d.eabs_e = float(p->eabs_e);
   d.eabs_g = float(p->eabs_g);
   d.wcc = float(p->wcc);
@@ -557,14 +550,14 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
     d64.x_lg2 = inv * std::log(2.0);
     d64.x_lo = -std::log(t.e_lo) * inv;
     const double *ph64, *el64;
-    if ((rc = upload(c, padded(t.ph_64), &ph64)) || (rc = upload(c, pairs_of(t.ph_64), &d64.mu)) ||
-        (rc = upload(c, padded(t.el_64), &el64)) ||
+    if ((rc = upload(c, t.ph_64, &ph64)) || (rc = upload(c, pairs_of(t.ph_64), &d64.mu)) ||
+        (rc = upload(c, t.el_64, &el64)) ||
         (rc = upload(c, t.pmol_64, &d64.pmol)))
       return rc;
     d64.ph = reinterpret_cast<const Dbl4 *>(ph64);
     d64.el = reinterpret_cast<const Dbl4 *>(el64);
     auto samp64 = [&](const std::vector<double> &v, int ne, double lo, double hi, SampTabT<double> &s) {
-      s.x_top = double(ne - 1) - double(1e-3f);
+      s.x_top = grid_top<double>(ne);
       s.nu = t.nu;
       s.y_top = double(t.nu - 1);
       s.lnE0 = std::log(lo);
@@ -582,7 +575,7 @@ int dpm_build_tables(dpm_ctx *c, const dpm_material *mats, int n_mat, const dpm_
     d64.msc_inv_dx = (t.msc_n - 1) / (t.msc_x1 - t.msc_x0);
     d64.msc_top = double(t.msc_n - 1);
     d64.msc_x1 = d64.msc_x0 + d64.msc_top / d64.msc_inv_dx;
-    d64.x_top = double(t.n_e - 1) - double(1e-3f);
+    d64.x_top = grid_top<double>(t.n_e);
     d64.eabs_e = p->eabs_e;
     d64.eabs_g = p->eabs_g;
     d64.wcc = p->wcc;

@@ -21,7 +21,6 @@ __global__ void k_diag_table(DevTables T, DevPhantom P, int which, int mat, int 
   if (i >= n) return;
   const float e = float(E[i]);
   const EIdx x = eidx(T, e);
-  const int next = min(x.i + 1, T.n_e - 1);  // the position's upper clamp may be the last node itself (n_e > 32769)
   double r = 0.0;
   switch (which) {
     case 0: r = ph_at(T, mat, x).x; break;
@@ -31,13 +30,13 @@ __global__ void k_diag_table(DevTables T, DevPhantom P, int which, int mat, int 
     case 4: r = el_at(T, mat, x).y; break;
     case 5: r = el_at(T, mat, x).z; break;
     case 6: r = el_at(T, mat, x).w; break;
-    case 7: r = lerp(T.pmol[size_t(mat) * T.n_e + x.i], T.pmol[size_t(mat) * T.n_e + next], x.f); break;
+    case 7: r = lerp(T.pmol[size_t(mat) * T.n_e + x.i], T.pmol[size_t(mat) * T.n_e + x.i + 1], x.f); break;
     case 8: {
       const float4 a = el_at(T, mat, x);
       r = csda_energy(T, mat, e, Held{a.x, a.y}, float(aux[i]));
       break;
     }
-    case 9: r = lerp(P.mu_max[x.i], P.mu_max[next], x.f); break;
+    case 9: r = lerp(P.mu_max[x.i], P.mu_max[x.i + 1], x.f); break;
     default: r = 0.0;
   }
   out[i] = r;

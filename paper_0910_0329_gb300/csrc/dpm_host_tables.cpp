@@ -27,7 +27,7 @@ void dpm_host_tables_free(void *h) { delete static_cast<dpm::HostTables *>(h); }
 int dpm_host_tables_get(void *h, const char *name, float *out, int n, double *meta) {
   const dpm::HostTables &t = *static_cast<dpm::HostTables *>(h);
   const std::vector<float> *v = nullptr;
-  double m[6] = {t.e_lo, t.e_hi, double(t.n_e), 0, 0, double(t.nu)};
+  double m[6] = {t.e_lo, t.e_hi, double(t.n_e), 0, double(dpm::grid_top<float>(t.n_e)), double(t.nu)};
   if (!std::strcmp(name, "ph")) v = &t.ph;
   else if (!std::strcmp(name, "el")) v = &t.el;
   else if (!std::strcmp(name, "pmol")) v = &t.pmol;

@@ -2,6 +2,8 @@
 // the kernels and the C ABI.  Nothing here is part of the public interface.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -41,6 +43,14 @@ struct Vec4<double> {
   using type = Dbl4;
 };
 
+// Largest position on a grid of n nodes that an interpolation takes: 1e-3 below the
+// last node, or the next number below it where 1e-3 is less than half an ulp (FP32
+// from 32770 nodes up), so that the node after it is always one of the grid's.
+template <class Real>
+inline Real grid_top(int n) {
+  return std::min(Real(n - 1) - Real(1e-3f), std::nextafter(Real(n - 1), Real(0)));
+}
+
 // One inverse-CDF sampling table: rows on a uniform ln(E) grid, columns on a
 // uniform grid in the uniform deviate u; entries are a normalised variable in
 // [0, 1] whose meaning depends on the process (see dpm_tables.cpp).
@@ -48,7 +58,7 @@ template <class Real>
 struct SampTabT {
   const Real *y;  // [ne][nu]
   int nu;
-  Real x_top, y_top;  // largest energy position (ne - 1 - 1e-3), nu - 1
+  Real x_top, y_top;  // largest energy position (grid_top), nu - 1
   Real lnE0, inv_dlnE;
 };
 
@@ -62,8 +72,8 @@ struct DevTablesT {
   int n_mat, n_e;
   Real lnE_lo, inv_dlnE;
   Real x_lg2, x_lo;  // grid position = log2(E) * x_lg2 + x_lo
-  Real x_top;        // largest position, n_e - 1 - 1e-3
-  // per-material tables [n_mat][n_e], and one node more
+  Real x_top;        // largest position (grid_top)
+  // per-material tables [n_mat][n_e]
   const V4 *ph;    // {mu/rho total (cm^2/g), Compton fraction, photoelectric fraction, 0}
   const Real *mu;  // the first component alone, [n_mat][n_e][2]: value, difference to the next node (0 at the last)
   const V4 *el;    // {R (g/cm^2), S (MeV cm^2/g), Sigma_hard (cm^2/g), 1/lambda1 (cm^2/g)}
