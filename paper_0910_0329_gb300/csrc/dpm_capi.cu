@@ -632,10 +632,12 @@ int dpm_update_phantom(dpm_ctx *c, int id, const uint8_t *mat, const float *rho)
   if (!p) return fail(c, DPM_EINVAL, "bad phantom id");
   if (!mat || !rho) return fail(c, DPM_EINVAL, "null pointer");
   cudaSetDevice(c->device);
-  // The arrays are staged in the batch slabs, which hold nothing between runs
-  // (or, before the first run, in the tally, which is zero then), so that an
-  // invalid array leaves the phantom as it was.
+  // The arrays are staged in the batch slabs, which hold nothing between runs, so
+  // that an invalid array leaves the phantom as it was; without slabs in the tally,
+  // which is zero before the first run.  A tally without slabs (a run that found no
+  // room for larger ones) is given up only once the host has found the arrays valid.
   int rc;
+  if (!p->d_slabs && p->n_total != 0 && (rc = scan_phantom(c, mat, rho, p->V))) return rc;
   if ((rc = upload_voxels(c, p, mat, rho, p->d_slabs ? static_cast<void *>(p->d_slabs) : p->d_S1))) {
     if (!p->d_slabs) CUDA_TRY(c, cudaMemsetAsync(p->d_S1, 0, p->V * sizeof(long long), c->stream));
     return rc;
