@@ -403,7 +403,11 @@ int dpm_diag_table(dpm_ctx *ctx, int which, int mat, int n, const double *energy
    unit vector (0.36, -0.48, 0.8) (aux 0..2) or +z (aux 3..5) turned by polar
    cosine e and azimuth 2 pi u, its component int(aux) % 3, 8 path from
    x = u cm to the far face of a 1 cm voxel [0, 1) along direction cosine e,
-   9 Sauter's 1 - cos(theta) of a photoelectron of kinetic energy e. */
+   9 Sauter's 1 - cos(theta) of a photoelectron of kinetic energy e.
+   10 to 19 are the single-precision functions of the transport: 10 1/u, 11 e/u,
+   12 the square root of u, 13 u truncated to an integer and 14 to a float, 15 the
+   face below (aux 0) or above (aux 1) voxel u in voxels, 16 log2 u, 17 exp u,
+   18 1/sqrt(u), 19 the hardware quotient e/u. */
 int dpm_diag_sample(dpm_ctx *ctx, int which, double e, double aux, int n, const double *u, double *out);
 
 /* n Philox4x32-10 blocks for counters ctr[4*i..] and keys key[2*i..] (host). */

@@ -98,6 +98,21 @@ __global__ void k_diag_sample(DevTables T, int which, float e, float aux, int n,
       break;
     }
     case 9: r = sauter_nu(T, e, lnE, x); break;
+    case 10: r = Num<float>::rcp(x); break;
+    case 11: r = Num<float>::div(e, x); break;
+    case 12: r = Num<float>::sqrt(x); break;
+    case 13:
+    case 14: {
+      float f;
+      const int k = Num<float>::trunc(x, &f);
+      r = which == 13 ? double(k) : double(f);
+      break;
+    }
+    case 15: r = Num<float>::face(uint32_t(x), aux > 0.5f); break;
+    case 16: r = Num<float>::log2_hw(x); break;
+    case 17: r = Num<float>::exp_hw(x); break;
+    case 18: r = Num<float>::rsqrt(x); break;
+    case 19: r = Num<float>::div_hw(e, x); break;
     default: r = 0.0;
   }
   out[i] = r;
