@@ -113,16 +113,20 @@ class Server:
         """Device bytes counted against the budget now: fixed part and slots."""
         return self.fixed + self.srv.info()["slot_bytes"]
 
-    def _collect(self, waiting, admitted_by, now):
-        """Statuses after a round: admission times, progress, and the done
-        requests' results (their slots are released)."""
+    def _admitted(self, waiting, now):
+        """Admission time of the requests that have got their slot by now."""
+        for rid, r in waiting.items():
+            if r.admitted is None and self.srv.status(rid)["state"] != dpm.REQ_PENDING:
+                r.admitted = now
+
+    def _collect(self, waiting, now):
+        """Statuses after a round: progress, and the done requests' results
+        (their slots are released)."""
         for rid in list(waiting):
             r = waiting[rid]
             st = self.srv.status(rid)
             if st["state"] == dpm.REQ_PENDING:
                 continue
-            if r.admitted is None:
-                r.admitted = admitted_by
             r.slot, r.histories, r.rounds = st["slot"], st["histories"], st["rounds"]
             r.rel_sigma, r.dose_max = st["rel_sigma"], st["dose_max"]
             if st["state"] == dpm.REQ_DONE:
@@ -160,15 +164,18 @@ class Server:
                 # requests that arrive while the round is on the GPU get their
                 # slots meanwhile
                 ran = self.srv.round_begin()
+                self._admitted(waiting, now)
                 while i < len(todo) and not self.srv.round_ready():
-                    if arrivals()[1]:
+                    now, new = arrivals()
+                    if new:
                         self.srv.admit()
+                        self._admitted(waiting, now)
                 self.srv.round_end()
                 if not ran and self.srv.info()["n_pending"]:
                     # nothing active and still nothing admissible, with every
                     # released slot free to go
                     raise RuntimeError("a request does not fit the HBM budget")
-                self._collect(waiting, now, clock())
+                self._collect(waiting, clock())
             else:
                 time.sleep(max(0.0, (todo[i].arrival - clock()) / time_scale))
         info = self.srv.info()
