@@ -164,13 +164,15 @@ class Server:
                 # requests that arrive while the round is on the GPU get their
                 # slots meanwhile
                 ran = self.srv.round_begin()
-                self._admitted(waiting, now)
-                while i < len(todo) and not self.srv.round_ready():
-                    now, new = arrivals()
-                    if new:
-                        self.srv.admit()
-                        self._admitted(waiting, now)
-                self.srv.round_end()
+                try:
+                    self._admitted(waiting, now)
+                    while i < len(todo) and not self.srv.round_ready():
+                        now, new = arrivals()
+                        if new:
+                            self.srv.admit()
+                            self._admitted(waiting, now)
+                finally:  # no round stays in flight, whatever a request's arrival raised
+                    self.srv.round_end()
                 if not ran and self.srv.info()["n_pending"]:
                     # nothing active and still nothing admissible, with every
                     # released slot free to go

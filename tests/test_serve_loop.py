@@ -88,3 +88,15 @@ def test_no_request_is_admitted_before_it_arrives(server, arrivals):
     if len(arrivals) > 1 and arrivals[1] == 3.5:
         r = next(r for r in st.completed if r.rid == 1)
         assert r.admitted - r.arrival <= 2 * POLL
+
+
+def test_an_error_during_a_round_leaves_none_in_flight(server):
+    submit = server.srv.submit
+    server.srv.submit = lambda g, source, seed: submit(g, source, seed) if seed != 1 else 1 / 0
+    with pytest.raises(ZeroDivisionError):
+        server.run(requests(0.0, 3.5), clock=lambda: server.srv.t)
+    assert server.srv.n_rounds == 1
+    server.srv.submit = submit
+    t0 = server.srv.t
+    st = server.run(requests(0.0), clock=lambda: server.srv.t - t0)
+    assert len(st.completed) == 1
