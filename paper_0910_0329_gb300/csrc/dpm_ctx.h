@@ -84,7 +84,7 @@ struct dpm_ctx {
   dpm::DevJob *d_jobs = nullptr;               // job table, kMaxJobs entries
   dpm::DmaxOut dmax;        // dpm_dmax_sigma results
   dpm::DmaxOut round_dmax;  // those of the server round in flight
-  const void *round_of = nullptr;  // the server whose round is in flight
+  std::weak_ptr<void> round;       // held by the server whose round is in flight
   unsigned long long *d_batch_counters = nullptr;  // [kCounterSlots]
   std::vector<cudaEvent_t> batch_ev;           // start/end pairs since the last dpm_batch_stats
   double batch_folded_ms = 0;                  // times of pairs retired early (see kMaxPendingEvents)

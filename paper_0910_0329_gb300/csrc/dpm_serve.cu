@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <cmath>
 #include <deque>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -60,6 +61,7 @@ struct dpm_server {
   std::deque<int> pending;           // ids in submission order
   std::vector<int> active;           // ids in admission order
   std::vector<int> chosen;           // ids of the round in flight
+  std::shared_ptr<void> round;       // held while it is (dpm_ctx::round)
   std::vector<Geometry> geom;        // by geometry phantom id
   std::vector<int> slot_geometry;    // by phantom id: the geometry a slot copies (-1: not a slot)
   uint64_t used = 0;                 // device bytes held by slots
@@ -197,9 +199,8 @@ int dpm_server_create(dpm_ctx *ctx, const dpm_serve_opts *opts, dpm_server **out
 }
 
 void dpm_server_destroy(dpm_server *s) {
-  if (!s) return;
-  // the slots stay loaded phantoms of the context (freed with it)
-  if (!s->chosen.empty()) s->ctx->round_of = nullptr;  // a round in flight ends unread
+  // the slots stay loaded phantoms of the context (freed with it, which may have
+  // happened by now); a round in flight ends unread
   delete s;
 }
 
@@ -248,7 +249,7 @@ int dpm_server_admit(dpm_server *s) {
 int dpm_server_round_begin(dpm_server *s, int *n_jobs) {
   if (!s) return DPM_EINVAL;
   if (n_jobs) *n_jobs = 0;
-  if (s->ctx->round_of) return srv_fail(s, DPM_ESTATE, "a round is in flight on the context");
+  if (!s->ctx->round.expired()) return srv_fail(s, DPM_ESTATE, "a round is in flight on the context");
   int rc = admit(s);
   if (rc) return rc;
   if (s->active.empty()) return DPM_OK;
@@ -275,7 +276,8 @@ int dpm_server_round_begin(dpm_server *s, int *n_jobs) {
   if ((rc = dpm_run_batch(s->ctx, jobs.data(), int(jobs.size()), &ro))) return rc;
   if ((rc = ctx_dmax_launch(s->ctx, s->ctx->round_dmax, slots.data(), int(slots.size())))) return rc;
   s->chosen.swap(chosen);
-  s->ctx->round_of = s;
+  s->round = std::make_shared<int>(0);
+  s->ctx->round = s->round;
   if (n_jobs) *n_jobs = k;
   return DPM_OK;
 }
@@ -296,7 +298,7 @@ int dpm_server_round_end(dpm_server *s, int *n_completed) {
   if (s->chosen.empty()) return DPM_OK;
   std::vector<int> chosen;
   chosen.swap(s->chosen);
-  s->ctx->round_of = nullptr;
+  s->round.reset();
   int rc = DPM_OK;
   std::vector<double> res(3 * chosen.size());
   if ((rc = ctx_dmax_read(s->ctx, s->ctx->round_dmax, int(chosen.size()), res.data()))) return rc;
