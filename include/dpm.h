@@ -117,10 +117,10 @@ typedef struct {
                           The kernels other than DPM_KERNEL_QUEUE are dpm_run only
                           (DPM_EINVAL elsewhere or for other values). */
     int n_batches;     /* history batches for the sigma estimate (default 50, max 1024) */
-    int block_size;    /* per-history kernel: threads per block (multiple of 32; 0 = 128).
-                          The queue kernel always runs blocks of 128 threads (it schedules
-                          per warp); its size is set by blocks_per_sm */
-    int blocks_per_sm; /* queue kernel: resident blocks per SM (0 = as many as fit, 6) */
+    int block_size;    /* not used: every transport kernel runs blocks of 128 threads (the
+                          queue kernel schedules per warp); the queue kernel's size is set
+                          by blocks_per_sm */
+    int blocks_per_sm; /* queue kernel: resident blocks per SM (0 = as many as fit) */
     int queue_log2;    /* queue kernel: log2 of each queue shard's capacity (7..20; 0 = 15 for
                           an electron-beam dpm_run, 14 otherwise) */
     int refill_min;    /* queue kernel: idle lanes before a warp takes particles from its
@@ -137,7 +137,7 @@ typedef struct {
                           graph and replay it while the batch keeps its shape */
     int count_events;  /* queue kernel: 1 = also count electron steps, photon flights and
                           interactions, tally atomics and secondaries for dpm_run_stats
-                          (about 10 % slower); 0 = those counts read 0.  The energy
+                          (8 to 9 % slower); 0 = those counts read 0.  The energy
                           counters and the tally are the same either way.  The per-history
                           kernels always count. */
     int refill_pause;  /* queue kernel: a warp with particles that found none to fetch
@@ -326,7 +326,8 @@ typedef struct {
 /* A server on ctx (opts may be NULL: all defaults; target_rel_sigma must then
    be set, so NULL gives DPM_EINVAL).  DPM_EINVAL for invalid options. */
 int dpm_server_create(dpm_ctx *ctx, const dpm_serve_opts *opts, dpm_server **server);
-/* Frees the server's host state; its slots stay phantoms of the context. */
+/* Frees the server's host state; its slots stay phantoms of the context (which
+   may be gone by then), and a round in flight ends unread. */
 void dpm_server_destroy(dpm_server *server);
 /* Queue a request on geometry_id (a loaded phantom, not a slot); *request_id
    numbers requests from 0 in submission order.  The source is copied.
@@ -467,7 +468,7 @@ int dpm_diag_atomic_replay(dpm_ctx *ctx, const uint32_t *ids, uint64_t n, uint64
    (emitted, escaped and missed energy, steps, flights, atomics, pushes, error
    flags) with `deposited` set to NaN: the deposited energy is the increase of
    the caller's d_tally times 2^-32 MeV.  With stats given the kernel also
-   counts events (dpm_run_opts.count_events), about 10 % slower; the tally is
+   counts events (dpm_run_opts.count_events), 8 to 9 % slower; the tally is
    the same either way. */
 #define DPM_NOALLOC_SCRATCH_BYTES (48u << 20)
 int dpm_run_noalloc(dpm_ctx *ctx, int phantom_id, const dpm_source *src, uint64_t first_history,

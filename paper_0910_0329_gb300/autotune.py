@@ -16,7 +16,7 @@ import os
 
 DEFAULT_SPACE = {
     "queue_log2": [12, 13, 14, 15],
-    "blocks_per_sm": [4, 6, 8],  # 6 fit, more are the same
+    "blocks_per_sm": [4, 6, 8],  # 7 fit: 8 takes as many as there is room for
     "refill_min": [0, 8, 16, 24],  # 0: the library's default (2 lanes)
     "refill_pause": [0, -1, 1],  # 0: the library's choice by queue size
 }

@@ -137,9 +137,9 @@ __device__ __forceinline__ void run_stack(const RunParamsT<Real> &R, Sink &s) {
   }
 }
 
-// 8 resident blocks of 128 threads cap the registers at 64, as in the queue
-// kernel: the extra spills cost less than the doubled occupancy gains
-// (+26 % on 6 MV, +30 % on 20 MeV electrons against 128 registers).
+// 8 resident blocks of 128 threads cap the registers at 64: the extra spills cost
+// less than the doubled occupancy gains (+26 % on 6 MV, +30 % on 20 MeV electrons
+// against 128 registers).
 template <class Real>
 __global__ void __launch_bounds__(128, 8) k_history(const __grid_constant__ RunParamsT<Real> R, uint64_t batch_size) {
   PartT<Real> stack[kHistStack];
