@@ -118,17 +118,21 @@ __device__ __forceinline__ void run_stack(const RunParamsT<Real> &R, Sink &s) {
     PartT<Real> q = s.stack[--s.sp];
     const bool photon = q.type == PHOTON;
     uint32_t cap = photon ? kMaxPhotonBlocks : kMaxElectronBlocks;
+    Real E_seen = q.E;
     EmissionT<Real> o;
     for (;;) {
       o.kind = EM_NONE;
-      const Real E0 = q.E;
       const bool alive = (q.type & CHAIN)      ? chain_step(q, R, s, o)
                          : photon              ? photon_flight(q, R, s, o)
                                                : electron_step(q, R, s, o);
       if (o.kind != EM_NONE && settle(q, o, R, s)) s.push(q, o);
       if (!alive) break;
-      if (photon && q.E != E0) cap = q.ctr + kMaxPhotonBlocks;  // scattered: as many again
       if (q.ctr >= cap) {
+        if (photon && q.E != E_seen) {  // a photon that has scattered since: as many again
+          E_seen = q.E;
+          cap += kMaxPhotonBlocks;
+          continue;
+        }
         s.error(ERR_STEPCAP);
         s.deposit(vox(q, R.P), q.E);
         break;

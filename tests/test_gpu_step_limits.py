@@ -36,3 +36,21 @@ def test_photons_between_whose_collisions_lie_many_virtual_ones():
         _, _, raw, st = d.read(pid)
     assert st["n_g_flights"] / 300 > 80_000
     assert raw.sum() / 2.0 ** 32 + st["escaped"] == pytest.approx(st["emitted"], rel=1e-9)
+
+
+def test_photons_that_need_their_limit_more_than_once():
+    """At twice that density some photons take more blocks in all than they may between
+    two scatters."""
+    ph = W.slab_phantom(40, 40, 40, 3.0, [(0, 1e9, W.MAT_WATER, 1.0)])
+    ph.rho[0] = 24000.0
+    src = W.Source(W.PHOTON, W.SPEC_MONO, 1.0, (60.0, 60.0, 0.0), 100.0, 1.0, 1.0)
+    out = []
+    with dpm.Dpm(0, W.MATERIALS, W.DEFAULT_PARAMS) as d:
+        for runs in ([(0, 300)], [(0, 113), (113, 187)]):
+            pid = d.load_phantom(ph)
+            for first, n in runs:
+                d.run(pid, src, n, 5, first=first, kernel=dpm.KERNEL_HISTORY)
+            _, _, raw, st = d.read(pid)  # raises on the step limit
+            assert st["n_histories"] == 300 and st["n_g_flights"] / 300 > 160_000
+            out.append(raw)
+    assert out[0].any() and np.array_equal(*out)
